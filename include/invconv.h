@@ -203,6 +203,26 @@ int invconv_backward_ws(const float* grad_x, const float* x, const float* w,
                         int B, int C, int H, int W, int k,
                         void* workspace, size_t workspace_bytes, void* stream);
 
+/* The same for the calls with the log-det folded in (scratch: invconv_workspace_bytes), the flow step
+ * (invconv_flow_step_workspace_bytes, one value for both directions) and the masked convolution
+ * (masked_conv_workspace_bytes; 0 where the call needs none): same rules, so one workspace of the largest size
+ * serves every call a program makes on a stream. */
+int invconv_forward_logdet_ws(const float* y, const float* w, float* x, float* logdet, int B, int C, int H, int W, int k,
+                              void* workspace, size_t workspace_bytes, void* stream);
+int invconv_backward_logdet_ws(const float* grad_x, const float* x, const float* w, const float* grad_logdet,
+                               float* grad_y, float* grad_w, int B, int C, int H, int W, int k,
+                               void* workspace, size_t workspace_bytes, void* stream);
+size_t invconv_flow_step_workspace_bytes(int B, int C, int H, int W, int k);
+int invconv_flow_step_forward_ws(const float* y, const float* w, const float* s, const float* b, const float* V,
+                                 float* x, float* u, float* logdet, int B, int C, int H, int W, int k,
+                                 void* workspace, size_t workspace_bytes, void* stream);
+int invconv_flow_step_backward_ws(const float* grad_u, const float* x, const float* w, const float* s, const float* b,
+                                  const float* V, float* grad_y, float* grad_w, float* grad_s, float* grad_b, float* grad_V,
+                                  int B, int C, int H, int W, int k, void* workspace, size_t workspace_bytes, void* stream);
+size_t masked_conv_workspace_bytes(int B, int C, int H, int W, int k);
+int masked_conv_forward_ws(const float* x, const float* w, float* y, int B, int C, int H, int W, int k,
+                           void* workspace, size_t workspace_bytes, void* stream);
+
 /* One whole layer step from HOST buffers: copies y, w, grad_x to the device,
  * runs invconv_forward, invconv_backward and invconv_logdet there, and copies
  * x, grad_y, grad_w and the log-det back -- enqueued on `stream`, no

@@ -1,7 +1,9 @@
-"""Thin ctypes binding of libinvconv_b200.so: argument marshalling only.
+"""Thin binding of libinvconv_b200.so: argument marshalling only.
 
 Function names mirror the C ABI in `include/invconv.h`.  torch supplies device
 memory and streams; every step of the computation runs inside the CUDA library.
+The calls on tensors go through the extension module `_native`
+(csrc/native_binding.cpp), the others through ctypes.
 There is no CPU or eager fallback: if the shared library is missing or a call
 returns a non-zero status, an exception is raised.
 """
@@ -21,6 +23,8 @@ PATH_AUTO, PATH_GENERIC, PATH_WARP, PATH_TEAM, PATH_TENSOR = range(5)
 WS_CONTROL_BYTES = 256
 
 _lib = None
+_native_ = None          # the extension module
+_bound_to = None         # the library its functions are bound to
 
 
 class InvConvError(RuntimeError):
@@ -99,6 +103,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def native():
+    """The extension module behind the tensor entry points, bound to the library that is loaded now."""
+    if _bound_to is None or _bound_to is not _lib:
+        _bind_native()
+    return _native_
+
+
+def _bind_native() -> None:
+    global _native_, _bound_to
+    from . import _native
+    L = lib()
+    _native.bind(tuple(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _native.names()), InvConvError)
+    _native_, _bound_to = _native, L
+
+
 def _check(status: int, what: str) -> None:
     if status != OK:
         raise InvConvError(status, what)
@@ -123,62 +142,17 @@ def _kern(w: torch.Tensor, C: int) -> int:
     return int(w.shape[2])
 
 
-_workspaces: dict = {}
-
-
-def workspace(B: int, C: int, H: int, W: int, k: int, device, stream_ptr: int, bf16: bool = False) -> Optional[torch.Tensor]:
-    """A zero-initialised scratch tensor for this shape, cached per (device, stream); `bf16`: sized for the
-    bfloat16-storage calls."""
-    size_of = lib().invconv_bf16_workspace_bytes if bf16 else lib().invconv_workspace_bytes
-    need = int(size_of(B, C, H, W, k))
-    if need == 0:
-        return None
-    key = (torch.device(device).index, stream_ptr)
-    ws = _workspaces.get(key)
-    if ws is None or ws.numel() < need:
-        ws = torch.zeros(need, dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-    return ws
-
-
 def invconv_forward(y: torch.Tensor, w: torch.Tensor, out: Optional[torch.Tensor] = None,
                     stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """x = f^{-1}(y).  y [B,C,H,W], w [C,C,k,k]  ->  x [B,C,H,W]."""
-    _act(y, "y")
-    B, C, H, W = y.shape
-    k = _kern(w, C)
-    x = torch.empty_like(y) if out is None else _act(out, "out")
-    with torch.cuda.device(y.device):
-        sp = _stream_ptr(stream, y.device)
-        ws = workspace(B, C, H, W, k, y.device, sp)
-        _check(lib().invconv_forward_ws(y.data_ptr(), w.data_ptr(), x.data_ptr(), B, C, H, W, k,
-                                        ws.data_ptr() if ws is not None else None,
-                                        ws.numel() if ws is not None else 0, sp), "invconv_forward")
-    return x
+    return native().forward(y, w, out, stream)
 
 
 def invconv_backward(grad_x: torch.Tensor, x: torch.Tensor, w: torch.Tensor, need_grad_w: bool = True,
                      out_grad_y: Optional[torch.Tensor] = None, out_grad_w: Optional[torch.Tensor] = None,
                      stream: Optional[torch.cuda.Stream] = None):
     """(grad_y, grad_w) through x = f^{-1}(y), given grad_x and the saved x."""
-    _act(grad_x, "grad_x")
-    _act(x, "x")
-    if grad_x.shape != x.shape:
-        raise ValueError("grad_x and x must have the same shape")
-    B, C, H, W = x.shape
-    k = _kern(w, C)
-    gy = torch.empty_like(grad_x) if out_grad_y is None else _act(out_grad_y, "out_grad_y")
-    gw = None
-    if need_grad_w:
-        gw = torch.empty_like(w) if out_grad_w is None else out_grad_w
-    with torch.cuda.device(x.device):
-        sp = _stream_ptr(stream, x.device)
-        ws = workspace(B, C, H, W, k, x.device, sp)
-        _check(lib().invconv_backward_ws(grad_x.data_ptr(), x.data_ptr(), w.data_ptr(), gy.data_ptr(),
-                                         gw.data_ptr() if gw is not None else None, B, C, H, W, k,
-                                         ws.data_ptr() if ws is not None else None,
-                                         ws.numel() if ws is not None else 0, sp), "invconv_backward")
-    return gy, gw
+    return native().backward(grad_x, x, w, need_grad_w, out_grad_y, out_grad_w, stream)
 
 
 NOALLOC_SCRATCH_BYTES = 1 << 20
@@ -204,14 +178,7 @@ def invconv_backward_noalloc(grad_x: torch.Tensor, x: torch.Tensor, w: torch.Ten
 def masked_conv_forward(x: torch.Tensor, w: torch.Tensor, out: Optional[torch.Tensor] = None,
                         stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """y = f(x), the sampling direction."""
-    _act(x, "x")
-    B, C, H, W = x.shape
-    k = _kern(w, C)
-    y = torch.empty_like(x) if out is None else _act(out, "out")
-    with torch.cuda.device(x.device):
-        _check(lib().masked_conv_forward(x.data_ptr(), w.data_ptr(), y.data_ptr(), B, C, H, W, k,
-                                         _stream_ptr(stream, x.device)), "masked_conv_forward")
-    return y
+    return native().conv(x, w, out, stream)
 
 
 def invconv_logdet(w: torch.Tensor, H: int, W: int, out: Optional[torch.Tensor] = None,
@@ -227,115 +194,39 @@ def invconv_logdet(w: torch.Tensor, H: int, W: int, out: Optional[torch.Tensor] 
 
 def invconv_forward_logdet(y: torch.Tensor, w: torch.Tensor, stream: Optional[torch.cuda.Stream] = None):
     """(x, logdet): x = f^{-1}(y) and the log-det of f in one call."""
-    _act(y, "y")
-    B, C, H, W = y.shape
-    k = _kern(w, C)
-    x = torch.empty_like(y)
-    ld = torch.empty(1, dtype=torch.float32, device=y.device)
-    with torch.cuda.device(y.device):
-        _check(lib().invconv_forward_logdet(y.data_ptr(), w.data_ptr(), x.data_ptr(), ld.data_ptr(), B, C, H, W, k,
-                                            _stream_ptr(stream, y.device)), "invconv_forward_logdet")
-    return x, ld
+    return native().forward_logdet(y, w, stream)
 
 
 def invconv_backward_logdet(grad_x: torch.Tensor, x: torch.Tensor, w: torch.Tensor, grad_logdet: torch.Tensor,
                             stream: Optional[torch.cuda.Stream] = None):
     """(grad_y, grad_w) with grad_logdet * d logdet / d w added to grad_w; grad_logdet is a one-element fp32
     CUDA tensor (the upstream gradient with respect to the log-det)."""
-    _act(grad_x, "grad_x")
-    _act(x, "x")
-    if grad_x.shape != x.shape:
-        raise ValueError("grad_x and x must have the same shape")
-    if grad_logdet.dtype != torch.float32 or grad_logdet.numel() != 1 or not grad_logdet.is_cuda:
-        raise ValueError("grad_logdet must be a one-element fp32 CUDA tensor")
-    B, C, H, W = x.shape
-    k = _kern(w, C)
-    gy, gw = torch.empty_like(grad_x), torch.empty_like(w)
-    with torch.cuda.device(x.device):
-        _check(lib().invconv_backward_logdet(grad_x.data_ptr(), x.data_ptr(), w.data_ptr(), grad_logdet.data_ptr(),
-                                             gy.data_ptr(), gw.data_ptr(), B, C, H, W, k,
-                                             _stream_ptr(stream, x.device)), "invconv_backward_logdet")
-    return gy, gw
+    return native().backward_logdet(grad_x, x, w, grad_logdet, stream)
 
 
 def invconv_flow_step_forward(y: torch.Tensor, w: torch.Tensor, s: torch.Tensor, b: torch.Tensor, V: torch.Tensor,
                               want_logdet: bool = True, stream: Optional[torch.cuda.Stream] = None):
     """(x, u, logdet) of one flow step: x = f^{-1}(y), u = V (s * x + b); logdet is a one-element tensor or None."""
-    _act(y, "y")
-    B, C, H, W = y.shape
-    k = _kern(w, C)
-    x, u = torch.empty_like(y), torch.empty_like(y)
-    ld = torch.empty(1, dtype=torch.float32, device=y.device) if want_logdet else None
-    with torch.cuda.device(y.device):
-        _check(lib().invconv_flow_step_forward(y.data_ptr(), w.data_ptr(), s.data_ptr(), b.data_ptr(), V.data_ptr(),
-                                               x.data_ptr(), u.data_ptr(), ld.data_ptr() if ld is not None else None,
-                                               B, C, H, W, k, _stream_ptr(stream, y.device)), "invconv_flow_step_forward")
-    return x, u, ld
+    return native().flow_forward(y, w, s, b, V, want_logdet, stream)
 
 
 def invconv_flow_step_backward(grad_u: torch.Tensor, x: torch.Tensor, w: torch.Tensor, s: torch.Tensor, b: torch.Tensor,
                                V: torch.Tensor, stream: Optional[torch.cuda.Stream] = None):
     """(grad_y, grad_w, grad_s, grad_b, grad_V) through one flow step, given grad_u and the saved x."""
-    _act(grad_u, "grad_u")
-    _act(x, "x")
-    B, C, H, W = x.shape
-    k = _kern(w, C)
-    gy, gw = torch.empty_like(x), torch.empty_like(w)
-    gs, gb, gV = torch.empty_like(s), torch.empty_like(b), torch.empty_like(V)
-    with torch.cuda.device(x.device):
-        _check(lib().invconv_flow_step_backward(grad_u.data_ptr(), x.data_ptr(), w.data_ptr(), s.data_ptr(), b.data_ptr(),
-                                                V.data_ptr(), gy.data_ptr(), gw.data_ptr(), gs.data_ptr(), gb.data_ptr(),
-                                                gV.data_ptr(), B, C, H, W, k, _stream_ptr(stream, x.device)),
-               "invconv_flow_step_backward")
-    return gy, gw, gs, gb, gV
-
-
-def _act16(t: torch.Tensor, name: str) -> torch.Tensor:
-    if not (t.is_cuda and t.dtype == torch.bfloat16 and t.dim() == 4 and t.is_contiguous()):
-        raise ValueError(f"{name} must be a contiguous bfloat16 CUDA tensor [B,C,H,W]")
-    return t
+    return native().flow_backward(grad_u, x, w, s, b, V, stream)
 
 
 def invconv_forward_bf16(y: torch.Tensor, w: torch.Tensor, out: Optional[torch.Tensor] = None,
                          stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """x = f^{-1}(y) with bfloat16 activations in memory (fp32 weights, fp32 arithmetic)."""
-    _act16(y, "y")
-    B, C, H, W = y.shape
-    k = _kern(w, C)
-    x = torch.empty_like(y) if out is None else _act16(out, "out")
-    with torch.cuda.device(y.device):
-        sp = _stream_ptr(stream, y.device)
-        if (y.data_ptr() | x.data_ptr()) & 15 or B == 0:
-            # buffers off a 16-byte boundary: the library sizes its own scratch for the route it has to take
-            _check(lib().invconv_forward_bf16(y.data_ptr(), w.data_ptr(), x.data_ptr(), B, C, H, W, k, sp), "invconv_forward_bf16")
-        else:
-            ws = workspace(B, C, H, W, k, y.device, sp, bf16=True)
-            _check(lib().invconv_forward_bf16_ws(y.data_ptr(), w.data_ptr(), x.data_ptr(), B, C, H, W, k,
-                                                 ws.data_ptr(), ws.numel(), sp), "invconv_forward_bf16")
-    return x
+    return native().forward_bf16(y, w, out, stream)
 
 
 def invconv_backward_bf16(grad_x: torch.Tensor, x: torch.Tensor, w: torch.Tensor, need_grad_w: bool = True,
                           out_grad_y: Optional[torch.Tensor] = None, out_grad_w: Optional[torch.Tensor] = None,
                           stream: Optional[torch.cuda.Stream] = None):
     """(grad_y, grad_w) with bfloat16 activations in memory; grad_w is fp32 (None if not asked for)."""
-    _act16(grad_x, "grad_x")
-    _act16(x, "x")
-    B, C, H, W = x.shape
-    k = _kern(w, C)
-    gy = torch.empty_like(x) if out_grad_y is None else _act16(out_grad_y, "out_grad_y")
-    gw = (out_grad_w if out_grad_w is not None else torch.empty_like(w)) if need_grad_w else None
-    with torch.cuda.device(x.device):
-        sp = _stream_ptr(stream, x.device)
-        gwp = gw.data_ptr() if gw is not None else None
-        if (grad_x.data_ptr() | x.data_ptr() | gy.data_ptr()) & 15 or B == 0:
-            _check(lib().invconv_backward_bf16(grad_x.data_ptr(), x.data_ptr(), w.data_ptr(), gy.data_ptr(), gwp,
-                                               B, C, H, W, k, sp), "invconv_backward_bf16")
-        else:
-            ws = workspace(B, C, H, W, k, x.device, sp, bf16=True)
-            _check(lib().invconv_backward_bf16_ws(grad_x.data_ptr(), x.data_ptr(), w.data_ptr(), gy.data_ptr(), gwp,
-                                                  B, C, H, W, k, ws.data_ptr(), ws.numel(), sp), "invconv_backward_bf16")
-    return gy, gw
+    return native().backward_bf16(grad_x, x, w, need_grad_w, out_grad_y, out_grad_w, stream)
 
 
 def invconv_bf16_in_kernel(B: int, C: int, H: int, W: int, k: int, backward: bool = False, with_grad_w: bool = True) -> bool:

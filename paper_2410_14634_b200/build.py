@@ -50,7 +50,9 @@ def _object_stale(obj: str, src: str) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every csrc/*.cu (one object each, in parallel) and link libinvconv_b200.so next to this file."""
+    """Compile every csrc/*.cu (one object each, in parallel) and link libinvconv_b200.so next to this file; the
+    extension module beside it."""
+    build_native(force)
     if not force and not _stale():
         return LIB
     objdir = os.path.join(PKG, "build")
@@ -74,6 +76,30 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC", *objs, "-o", tmp])
     os.replace(tmp, LIB)
     return LIB
+
+
+NATIVE = os.path.join(PKG, "_native.so")
+
+
+def build_native(force: bool = False) -> str:
+    """The Python extension module (csrc/native_binding.cpp), compiled against the installed torch."""
+    src = os.path.join(CSRC, "native_binding.cpp")
+    deps = [src, os.path.join(ROOT, "include", "invconv.h")]
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
+        return NATIVE
+    import sysconfig
+    import torch
+    base = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(NVCC))
+    inc = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"], os.path.join(ROOT, "include")]
+    libdir = os.path.join(base, "lib")
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                           *(f"-I{d}" for d in inc), src, "-o", tmp, f"-L{libdir}", f"-Wl,-rpath,{libdir}",
+                           "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10"])
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 LIB_DEBUG = os.path.join(PKG, "libinvconv_b200_debug.so")

@@ -265,24 +265,62 @@ int flow_bounds_info(int* info)
 
 }  // namespace invconv_internal
 
+namespace {
+
+// Scratch of a flow-step call: the layer's own workspace (its control words first), the gradient with respect to x where the
+// step is composed, and the shares of the parameter gradients.
+struct FlowScratch {
+    size_t layer, act, part, total;
+    int tiles, shares;
+};
+
+FlowScratch flow_scratch(int B, int C, int H, int W, int k)
+{
+    FlowScratch f;
+    f.layer = up256(invconv_workspace_bytes(B > 0 ? B : 1, C, H, W, k) + INVCONV_WS_CONTROL_BYTES);
+    f.act = up256(sizeof(float) * (size_t)B * C * H * W);
+    f.tiles = (H * W + kMixPixels - 1) / kMixPixels;
+    f.shares = invconv_internal::sm_count() * 2;
+    if (f.shares > B * f.tiles) f.shares = B * f.tiles;
+    if (f.shares < 1) f.shares = 1;
+    f.part = up256(sizeof(double) * ((size_t)C * C + C) * f.shares);
+    f.total = f.layer + f.act + f.part;
+    return f;
+}
+
+bool bad_shape(int B, int C, int H, int W, int k, int* rc)
+{
+    *rc = INVCONV_OK;
+    if (B < 0 || C < 1 || H < 1 || W < 1 || k < 1) *rc = INVCONV_BAD_ARG;
+    else if (k > INVCONV_MAX_K || C > INVCONV_MAX_C || (long long)B * C * H * W >= (1LL << 31)) *rc = INVCONV_UNSUPPORTED;
+    return *rc != INVCONV_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
-int invconv_flow_step_forward(const float* y, const float* w, const float* s, const float* b, const float* V,
-                              float* x, float* u, float* logdet, int B, int C, int H, int W, int k, void* stream)
+size_t invconv_flow_step_workspace_bytes(int B, int C, int H, int W, int k)
 {
-    if (B < 0 || C < 1 || H < 1 || W < 1 || k < 1) return INVCONV_BAD_ARG;
-    if (k > INVCONV_MAX_K || C > INVCONV_MAX_C) return INVCONV_UNSUPPORTED;
+    int rc;
+    if (bad_shape(B, C, H, W, k, &rc)) return 0;
+    return flow_scratch(B, C, H, W, k).total;
+}
+
+int invconv_flow_step_forward_ws(const float* y, const float* w, const float* s, const float* b, const float* V,
+                                 float* x, float* u, float* logdet, int B, int C, int H, int W, int k,
+                                 void* workspace, size_t workspace_bytes, void* stream)
+{
+    int rc;
+    if (bad_shape(B, C, H, W, k, &rc)) return rc;
     if (!w || !s || !b || !V) return INVCONV_BAD_ARG;
     if (B > 0 && (!y || !x || !u || y == x || u == x || u == y)) return INVCONV_BAD_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (B > 0) {
-        Scratch sc;
-        const size_t need = invconv_workspace_bytes(B, C, H, W, k);
-        const int ra = sc.acquire(need, st);
-        if (ra) return ra;
-        int rc = invconv_internal::warp_step_forward(y, w, s, b, V, x, u, Geom{B, C, H, W, k}, sc.p, st);
+        if (!workspace || workspace_bytes < flow_scratch(B, C, H, W, k).total) return INVCONV_WORKSPACE_TOO_SMALL;
+        rc = invconv_internal::warp_step_forward(y, w, s, b, V, x, u, Geom{B, C, H, W, k}, workspace, st);
         if (rc == INVCONV_UNSUPPORTED) {
-            rc = invconv_forward_ws(y, w, x, B, C, H, W, k, sc.p, need, stream);
+            rc = invconv_forward_ws(y, w, x, B, C, H, W, k, workspace, workspace_bytes, stream);
             if (rc) return rc;
             rc = launch_mix<false>(x, V, s, b, u, B, C, H * W, st);
         }
@@ -291,7 +329,7 @@ int invconv_flow_step_forward(const float* y, const float* w, const float* s, co
     if (logdet) {
         auto kern = flow_logdet_kernel;
         const size_t sm = sizeof(double) * (size_t)C * C;
-        const int rc = invconv_internal::set_smem_limit(kern, sm);
+        rc = invconv_internal::set_smem_limit(kern, sm);
         if (rc) return rc;
         kern<<<1, 128, sm, st>>>(w, s, V, logdet, C, H, W, k);
         return check_launch();
@@ -299,44 +337,45 @@ int invconv_flow_step_forward(const float* y, const float* w, const float* s, co
     return INVCONV_OK;
 }
 
-int invconv_flow_step_backward(const float* grad_u, const float* x, const float* w, const float* s, const float* b,
-                               const float* V, float* grad_y, float* grad_w, float* grad_s, float* grad_b, float* grad_V,
-                               int B, int C, int H, int W, int k, void* stream)
+int invconv_flow_step_forward(const float* y, const float* w, const float* s, const float* b, const float* V,
+                              float* x, float* u, float* logdet, int B, int C, int H, int W, int k, void* stream)
 {
-    if (B < 0 || C < 1 || H < 1 || W < 1 || k < 1) return INVCONV_BAD_ARG;
-    if (k > INVCONV_MAX_K || C > INVCONV_MAX_C) return INVCONV_UNSUPPORTED;
+    Scratch sc;
+    const size_t need = B > 0 ? invconv_flow_step_workspace_bytes(B, C, H, W, k) : 0;
+    const int ra = sc.acquire(need, reinterpret_cast<cudaStream_t>(stream));
+    if (ra) return ra;
+    return invconv_flow_step_forward_ws(y, w, s, b, V, x, u, logdet, B, C, H, W, k, sc.p, need, stream);
+}
+
+int invconv_flow_step_backward_ws(const float* grad_u, const float* x, const float* w, const float* s, const float* b,
+                                  const float* V, float* grad_y, float* grad_w, float* grad_s, float* grad_b, float* grad_V,
+                                  int B, int C, int H, int W, int k, void* workspace, size_t workspace_bytes, void* stream)
+{
+    int rc;
+    if (bad_shape(B, C, H, W, k, &rc)) return rc;
     if (!w || !s || !b || !V || !grad_w || !grad_s || !grad_b || !grad_V) return INVCONV_BAD_ARG;
     if (B > 0 && (!grad_u || !x || !grad_y || grad_u == grad_y || x == grad_y)) return INVCONV_BAD_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int HW = H * W;
-    const size_t act = up256(sizeof(float) * (size_t)B * C * HW);
-    const size_t need = up256(invconv_workspace_bytes(B > 0 ? B : 1, C, H, W, k) + INVCONV_WS_CONTROL_BYTES);
-    const int tiles = (HW + kMixPixels - 1) / kMixPixels;
-    int shares = invconv_internal::sm_count() * 2;
-    if (shares > B * tiles) shares = B * tiles;
-    if (shares < 1) shares = 1;
-    const size_t NE = (size_t)C * C + C;
-    const size_t part = up256(sizeof(double) * NE * shares);
-    Scratch sc;
-    const int ra = sc.acquire(need + act + part, st);
-    if (ra) return ra;
-    char* base = static_cast<char*>(sc.p);
-    float* grad_x = reinterpret_cast<float*>(base + need);
-    double* partials = reinterpret_cast<double*>(base + need + act);
-    int rc = INVCONV_OK;
+    const FlowScratch f = flow_scratch(B, C, H, W, k);
+    if (!workspace || workspace_bytes < f.total) return INVCONV_WORKSPACE_TOO_SMALL;
+    char* base = static_cast<char*>(workspace);
+    float* grad_x = reinterpret_cast<float*>(base + f.layer);
+    double* partials = reinterpret_cast<double*>(base + f.layer + f.act);
+    int shares = f.shares;
     if (B > 0) {
-        rc = invconv_internal::warp_step_backward(grad_u, x, w, s, V, grad_y, grad_w, Geom{B, C, H, W, k}, sc.p, st);
+        rc = invconv_internal::warp_step_backward(grad_u, x, w, s, V, grad_y, grad_w, Geom{B, C, H, W, k}, workspace, st);
         if (rc == INVCONV_UNSUPPORTED) {
             rc = launch_mix<true>(grad_u, V, s, b, grad_x, B, C, HW, st);
             if (rc) return rc;
-            rc = invconv_backward_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, sc.p, need, stream);
+            rc = invconv_backward_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, workspace, f.layer, stream);
         }
         if (rc) return rc;
         const size_t sm = sizeof(float) * 2 * (size_t)C * (kMixPixels + 1);
         auto kern = flow_mix_grad_kernel;
         rc = invconv_internal::set_smem_limit(kern, sm);
         if (rc) return rc;
-        kern<<<shares, 256, sm, st>>>(grad_u, x, partials, B, C, HW, tiles);
+        kern<<<shares, 256, sm, st>>>(grad_u, x, partials, B, C, HW, f.tiles);
         rc = check_launch();
         if (rc) return rc;
     } else {
@@ -344,12 +383,23 @@ int invconv_flow_step_backward(const float* grad_u, const float* x, const float*
         if (rc) return rc;
         shares = 0;
     }
-    const size_t smf = sizeof(double) * NE;
+    const size_t smf = sizeof(double) * ((size_t)C * C + C);
     auto kf = flow_mix_grad_final_kernel;
     rc = invconv_internal::set_smem_limit(kf, smf);
     if (rc) return rc;
     kf<<<1, 256, smf, st>>>(partials, shares, V, s, b, grad_V, grad_s, grad_b, C);
     return check_launch();
+}
+
+int invconv_flow_step_backward(const float* grad_u, const float* x, const float* w, const float* s, const float* b,
+                               const float* V, float* grad_y, float* grad_w, float* grad_s, float* grad_b, float* grad_V,
+                               int B, int C, int H, int W, int k, void* stream)
+{
+    Scratch sc;
+    const size_t need = invconv_flow_step_workspace_bytes(B, C, H, W, k);
+    const int ra = sc.acquire(need, reinterpret_cast<cudaStream_t>(stream));
+    if (ra) return ra;
+    return invconv_flow_step_backward_ws(grad_u, x, w, s, b, V, grad_y, grad_w, grad_s, grad_b, grad_V, B, C, H, W, k, sc.p, need, stream);
 }
 
 }  // extern "C"

@@ -1156,7 +1156,17 @@ int invconv_backward_bf16(const void* grad_x, const void* x, const float* w, voi
     return invconv_backward_bf16_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, sc.p, bytes, stream);
 }
 
-int masked_conv_forward(const float* x, const float* w, float* y, int B, int C, int H, int W, int k, void* stream)
+size_t masked_conv_workspace_bytes(int B, int C, int H, int W, int k)
+{
+    if (check_shape(B, C, H, W, k) != INVCONV_OK || B == 0) return 0;
+    const int forced = g_forced_path.load();
+    if (forced == INVCONV_PATH_GENERIC || forced == INVCONV_PATH_TEAM) return 0;
+    const ConvTensorPlan ct = plan_conv_tensor(B, C, H, W, k, kMaxDynSmem, sm_count());
+    return ct.ok ? INVCONV_WS_CONTROL_BYTES + ct.pack_bytes : 0;
+}
+
+int masked_conv_forward_ws(const float* x, const float* w, float* y, int B, int C, int H, int W, int k,
+                           void* workspace, size_t workspace_bytes, void* stream)
 {
     const int rc = check_shape(B, C, H, W, k);
     if (rc) return rc;
@@ -1166,12 +1176,12 @@ int masked_conv_forward(const float* x, const float* w, float* y, int B, int C, 
         const int rs = launch_masked_conv_small(x, w, y, Geom{B, C, H, W, k}, as_stream(stream));
         if (rs != INVCONV_UNSUPPORTED) return rs;
         // many channels: the tensor cores (forcing the team family keeps the FMA tile kernel, for comparison)
-        const ConvTensorPlan ct = plan_conv_tensor(B, C, H, W, k, kMaxDynSmem, sm_count());
-        if (ct.ok && g_forced_path.load() != INVCONV_PATH_TEAM) {
-            StreamScratch sc;
-            const int ra = sc.acquire(ct.pack_bytes, as_stream(stream));
-            if (ra) return ra;
-            return invconv_internal::conv_tensor_launch(ct, x, w, y, Geom{B, C, H, W, k}, static_cast<unsigned char*>(sc.p), as_stream(stream));
+        const size_t need = masked_conv_workspace_bytes(B, C, H, W, k);
+        if (need > 0) {
+            if (!workspace || workspace_bytes < need) return INVCONV_WORKSPACE_TOO_SMALL;
+            const ConvTensorPlan ct = plan_conv_tensor(B, C, H, W, k, kMaxDynSmem, sm_count());
+            return invconv_internal::conv_tensor_launch(ct, x, w, y, Geom{B, C, H, W, k},
+                                                        static_cast<unsigned char*>(workspace) + INVCONV_WS_CONTROL_BYTES, as_stream(stream));
         }
         const int rt = launch_masked_conv_tile(x, w, y, Geom{B, C, H, W, k}, as_stream(stream));
         if (rt != INVCONV_UNSUPPORTED) return rt;
@@ -1180,6 +1190,15 @@ int masked_conv_forward(const float* x, const float* w, float* y, int B, int C, 
     const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
     generic_masked_conv_kernel<<<blocks, 256, 0, as_stream(stream)>>>(x, w, y, Geom{B, C, H, W, k}, total);
     return check_launch();
+}
+
+int masked_conv_forward(const float* x, const float* w, float* y, int B, int C, int H, int W, int k, void* stream)
+{
+    StreamScratch sc;
+    const size_t need = (x && w && y && x != y) ? masked_conv_workspace_bytes(B, C, H, W, k) : 0;
+    const int ra = sc.acquire(need, as_stream(stream));
+    if (ra) return ra;
+    return masked_conv_forward_ws(x, w, y, B, C, H, W, k, sc.p, need, stream);
 }
 
 int invconv_logdet(const float* w, float* logdet, int C, int H, int W, int k, void* stream)
@@ -1191,24 +1210,33 @@ int invconv_logdet(const float* w, float* logdet, int C, int H, int W, int k, vo
     return check_launch();
 }
 
-int invconv_forward_logdet(const float* y, const float* w, float* x, float* logdet,
-                           int B, int C, int H, int W, int k, void* stream)
+int invconv_forward_logdet_ws(const float* y, const float* w, float* x, float* logdet, int B, int C, int H, int W, int k,
+                              void* workspace, size_t workspace_bytes, void* stream)
 {
     if (!logdet) return INVCONV_BAD_ARG;
     const int rc = check_shape(B, C, H, W, k);
     if (rc) return rc;
     if (!w) return INVCONV_BAD_ARG;
     if (B > 0 && (!y || !x || y == x)) return INVCONV_BAD_ARG;
-    StreamScratch sc;
     const int path = resolve_path(B > 0 ? B : 1, C, H, W, k);
     const size_t need = B > 0 ? workspace_bytes_for(path, B, C, H, W, k) : 0;
-    const int ra = sc.acquire(need, as_stream(stream));
-    if (ra) return ra;
-    return launch_forward(path, y, w, x, Geom{B, C, H, W, k}, sc.p, need, as_stream(stream), logdet);
+    if (need > 0 && (!workspace || workspace_bytes < need)) return INVCONV_WORKSPACE_TOO_SMALL;
+    return launch_forward(path, y, w, x, Geom{B, C, H, W, k}, workspace, workspace_bytes, as_stream(stream), logdet);
 }
 
-int invconv_backward_logdet(const float* grad_x, const float* x, const float* w, const float* grad_logdet,
-                            float* grad_y, float* grad_w, int B, int C, int H, int W, int k, void* stream)
+int invconv_forward_logdet(const float* y, const float* w, float* x, float* logdet,
+                           int B, int C, int H, int W, int k, void* stream)
+{
+    StreamScratch sc;
+    const size_t need = (logdet && w && check_shape(B, C, H, W, k) == INVCONV_OK && B > 0) ? invconv_workspace_bytes(B, C, H, W, k) : 0;
+    const int ra = sc.acquire(need, as_stream(stream));
+    if (ra) return ra;
+    return invconv_forward_logdet_ws(y, w, x, logdet, B, C, H, W, k, sc.p, need, stream);
+}
+
+int invconv_backward_logdet_ws(const float* grad_x, const float* x, const float* w, const float* grad_logdet,
+                               float* grad_y, float* grad_w, int B, int C, int H, int W, int k,
+                               void* workspace, size_t workspace_bytes, void* stream)
 {
     if (!grad_logdet || !grad_w) return INVCONV_BAD_ARG;
     const int rc = check_shape(B, C, H, W, k);
@@ -1224,12 +1252,21 @@ int invconv_backward_logdet(const float* grad_x, const float* x, const float* w,
         return check_launch();
     }
     if (!grad_x || !x || !grad_y || grad_x == grad_y || x == grad_y) return INVCONV_BAD_ARG;
-    StreamScratch sc;
     const int path = resolve_path(B, C, H, W, k);
     const size_t need = workspace_bytes_for(path, B, C, H, W, k);
+    if (need > 0 && (!workspace || workspace_bytes < need)) return INVCONV_WORKSPACE_TOO_SMALL;
+    return launch_backward(path, grad_x, x, w, grad_y, grad_w, Geom{B, C, H, W, k}, workspace, workspace_bytes, as_stream(stream), grad_logdet);
+}
+
+int invconv_backward_logdet(const float* grad_x, const float* x, const float* w, const float* grad_logdet,
+                            float* grad_y, float* grad_w, int B, int C, int H, int W, int k, void* stream)
+{
+    StreamScratch sc;
+    const bool args = grad_logdet && grad_w && w && grad_x && x && grad_y && check_shape(B, C, H, W, k) == INVCONV_OK && B > 0;
+    const size_t need = args ? invconv_workspace_bytes(B, C, H, W, k) : 0;
     const int ra = sc.acquire(need, as_stream(stream));
     if (ra) return ra;
-    return launch_backward(path, grad_x, x, w, grad_y, grad_w, Geom{B, C, H, W, k}, sc.p, need, as_stream(stream), grad_logdet);
+    return invconv_backward_logdet_ws(grad_x, x, w, grad_logdet, grad_y, grad_w, B, C, H, W, k, sc.p, need, stream);
 }
 
 size_t invconv_step_scratch_bytes(int B, int C, int H, int W, int k)
