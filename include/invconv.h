@@ -335,6 +335,7 @@ enum invconv_option {
     INVCONV_OPT_TEAM_VARIANT,        /* 0 (default): by shape; 1: channel-slice kernel; 2: pixel-team kernel */
     INVCONV_OPT_TEAM_CLUSTER,        /* 0 (default): by shape; 1..8: force the cluster size of the channel-slice kernel */
     INVCONV_OPT_DEPENDENT_LAUNCH,    /* 1 (default): programmatic dependent launch between the library's kernels; 0: off */
+    INVCONV_OPT_LINE,                /* -1 (default): by shape; 0: never the line wavefront (one thread per row and channel); 1: wherever it serves the shape */
     INVCONV_OPT_COUNT
 };
 int invconv_set_option(int option, int value);

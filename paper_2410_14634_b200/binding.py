@@ -267,13 +267,13 @@ class HostStep:
 
 # invconv_option values (development and test controls, see include/invconv.h)
 (OPT_WARP_RING, OPT_WARP_CHANNEL_SPLIT, OPT_GRADW_SEPARATE, OPT_GRADW_TENSOR_PIPE, OPT_TEAM_VARIANT,
- OPT_TEAM_CLUSTER, OPT_DEPENDENT_LAUNCH) = range(7)
+ OPT_TEAM_CLUSTER, OPT_DEPENDENT_LAUNCH, OPT_LINE) = range(8)
 
 
 def invconv_set_option(option: int, value: int) -> int:
     """Set a development/test control; returns the previous value."""
     prev = int(lib().invconv_set_option(option, value))
-    if prev == -1 and not (0 <= option < 7):
+    if prev == -1 and not (0 <= option < 8):
         raise ValueError("unknown option")
     return prev
 

@@ -112,7 +112,8 @@ def build_debug_bounds() -> str:
     objdir = os.path.join(PKG, "build")
     flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",
              "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-DINVCONV_DEBUG_BOUNDS"]
-    procs, objs = [], [os.path.join(objdir, "invconv_lib.o")]
+    procs, objs = [], [os.path.join(objdir, os.path.basename(src)[:-3] + ".o") for src in sources()
+                   if os.path.basename(src) not in ("tensor_lib.cu", "flow_step_lib.cu")]
     for name in ("tensor_lib", "flow_step_lib"):
         obj = os.path.join(objdir, name + "_dbg.o")
         objs.append(obj)

@@ -21,6 +21,7 @@
 #include "lib_internal.h"
 #include "gradw_kernels.cuh"
 #include "conv_kernels.cuh"
+#include "line_params.h"
 
 using namespace invconv;
 using invconv_internal::set_smem_limit;
@@ -31,7 +32,7 @@ namespace {
 std::atomic<int> g_forced_path{INVCONV_PATH_AUTO};
 std::atomic<unsigned long long> g_kernel_launches{0};
 // development and test controls (invconv_set_option); defaults as documented in the header
-std::atomic<int> g_opt[INVCONV_OPT_COUNT] = {{1}, {1}, {-1}, {1}, {0}, {0}, {1}};
+std::atomic<int> g_opt[INVCONV_OPT_COUNT] = {{1}, {1}, {-1}, {1}, {0}, {0}, {1}, {-1}};
 inline int opt(int o) { return g_opt[o].load(std::memory_order_relaxed); }
 
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
@@ -68,16 +69,6 @@ int check_shape(int B, int C, int H, int W, int k)
 // ---------------------------------------------------------------- warp family
 #define INVCONV_WARP_CASES(X) \
     X(1, 2) X(1, 3) X(1, 5) X(2, 2) X(2, 3) X(2, 5) X(3, 2) X(3, 3) X(3, 5) X(4, 2) X(4, 3) X(4, 5)
-
-struct WarpPlan {
-    bool ok = false;
-    bool glb = false;      // image too large for shared memory: operands stay in global memory
-    bool ring = false;     // ... and a ring of 128 columns per warp fits: streamed through shared memory
-    bool cs = false;       // channel-split walk available (lane = (row, output channel)); its own geometry below
-    int nb = 0, ipc = 0, grid = 0;
-    int nb_cs = 0, ipc_cs = 0, grid_cs = 0;
-    size_t smem = 0, smem_ring = 0, smem_cs = 0;
-};
 
 template <int C, int K>
 WarpPlan plan_warp_ck(int B, int H, int W, bool bwd)
@@ -128,49 +119,6 @@ WarpPlan plan_warp(int B, int C, int H, int W, int k, bool bwd)
     return WarpPlan{};
 }
 
-template <int C, int K, bool BWD>
-int launch_warp_ck(const WarpPlan& pl, WarpParams prm, cudaStream_t st)
-{
-    // global-memory mode: streamed through a shared-memory ring unless grad_w rides along in the wavefront
-    const bool ring = pl.glb && pl.ring && prm.grad_w == nullptr && opt(INVCONV_OPT_WARP_RING) != 0;
-    // channel-split walk (its own row-block geometry) unless grad_w rides along in the wavefront
-    bool cs = false;
-    if constexpr (C >= 3 && K == 5) cs = pl.cs && prm.grad_w == nullptr && opt(INVCONV_OPT_WARP_CHANNEL_SPLIT) != 0;
-    auto kern = ring ? warp_wavefront_kernel<C, K, BWD, true, true, true>
-                     : (pl.glb ? warp_wavefront_kernel<C, K, BWD, true, true>
-                               : (pl.nb > 1 ? warp_wavefront_kernel<C, K, BWD, true> : warp_wavefront_kernel<C, K, BWD, false>));
-    size_t smem = ring ? pl.smem_ring : pl.smem;
-    int nb = pl.nb, ipc = pl.ipc, grid = pl.grid;
-    if constexpr (C >= 3 && K == 5) {
-        if (cs) {
-            kern = pl.nb_cs > 1 ? warp_wavefront_kernel<C, K, BWD, true, false, false, true>
-                                : warp_wavefront_kernel<C, K, BWD, false, false, false, true>;
-            smem = pl.smem_cs; nb = pl.nb_cs; ipc = pl.ipc_cs; grid = pl.grid_cs;
-            prm.nb = nb; prm.ipc = ipc;
-        }
-    }
-    const int rc = set_smem_limit(kern, smem);
-    if (rc) return rc;
-    // Programmatic dependent launch: the kernel may be scheduled while its predecessor on the stream drains;
-    // it touches no global memory before griddepcontrol.wait, which waits for that predecessor to complete.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(nb * ipc * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = opt(INVCONV_OPT_DEPENDENT_LAUNCH) ? 1 : 0;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, prm);
-    if (e != cudaSuccess) {
-        std::fprintf(stderr, "invconv: warp launch failed: %s\n", cudaGetErrorString(e));
-        cudaGetLastError();
-        return INVCONV_CUDA_ERROR;
-    }
-    return check_launch();
-}
-
 constexpr size_t kGradWSmallSmem = 96 * 1024;
 
 using invconv_internal::sm_count;
@@ -196,30 +144,6 @@ bool gradw_separate(const WarpPlan& pl, const GradWSmallPlan& gs, int C, int k)
     return pl.glb || C * C * k * k > 81;
 }
 
-template <int C, int K>
-int launch_gradw_small_ck(const GradWSmallPlan& gs, const GradWSmallParams& prm, cudaStream_t st)
-{
-    auto kern = gradw_small_kernel<C, K>;
-    const int rc = set_smem_limit(kern, gs.smem);
-    if (rc) return rc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(gs.grid);
-    cfg.blockDim = dim3(GradWSmallShape<C, K>::NT);
-    cfg.dynamicSmemBytes = gs.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = opt(INVCONV_OPT_DEPENDENT_LAUNCH) ? 1 : 0;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, prm);
-    if (e != cudaSuccess) {
-        std::fprintf(stderr, "invconv: grad_w launch failed: %s\n", cudaGetErrorString(e));
-        cudaGetLastError();
-        return INVCONV_CUDA_ERROR;
-    }
-    return check_launch();
-}
-
 int launch_gradw_small(const GradWSmallPlan& gs, const float* gy, const float* x, float* gw, Geom g, void* ws, cudaStream_t st,
                        const LogdetFuse& ld)
 {
@@ -237,10 +161,14 @@ int launch_gradw_small(const GradWSmallPlan& gs, const float* gy, const float* x
     prm.div_rb = make_fast_div((unsigned)gs.RB);
     prm.div_xr = make_fast_div((unsigned)(gs.RB + g.k - 1));
     prm.div_qpr = make_fast_div((unsigned)(gs.gst / 4));
-#define X(CC, KK) if (g.C == CC && g.k == KK) return launch_gradw_small_ck<CC, KK>(gs, prm, st);
-    INVCONV_WARP_CASES(X)
-#undef X
-    return INVCONV_UNSUPPORTED;
+    const bool dep = opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0;
+    switch (g.C) {
+    case 1: return invconv_internal::launch_gradw_small_c1(g.k, gs, prm, dep, st);
+    case 2: return invconv_internal::launch_gradw_small_c2(g.k, gs, prm, dep, st);
+    case 3: return invconv_internal::launch_gradw_small_c3(g.k, gs, prm, dep, st);
+    case 4: return invconv_internal::launch_gradw_small_c4(g.k, gs, prm, dep, st);
+    default: return INVCONV_UNSUPPORTED;
+    }
 }
 
 // The per-pixel neighbours of the layer in a flow step, applied inside the wavefront kernel (see WarpParams).
@@ -250,6 +178,51 @@ struct WarpMix {
     bool grad_in = false;       // backward
 };
 
+// ---------------------------------------------------------------- line wavefront (one thread per row and channel)
+LinePlan line_plan(int B, int C, int H, int W, int k, bool bf16 = false)
+{
+    // bfloat16 images are walked in one band only: a band's halo rows come back from the output, where they would be rounded
+    return plan_line(B, C, H, W, k, kMaxDynSmem, sm_count(), bf16 ? 1 : 32);
+}
+
+bool line_preferred(int B, int C, int H, int W, int k);
+
+// The solve through the line wavefront; INVCONV_UNSUPPORTED where it has no plan.
+int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cudaStream_t st, const WarpMix* mix = nullptr,
+                float* logdet_out = nullptr, bool bf16 = false)
+{
+    const LinePlan pl = line_plan(g.B, g.C, g.H, g.W, g.k, bf16);
+    if (!pl.ok) return INVCONV_UNSUPPORTED;
+    LineParams prm = {};
+    prm.rhs = rhs; prm.w = w; prm.out = out;
+    prm.B = g.B; prm.C = g.C; prm.H = g.H; prm.W = g.W;
+    prm.HB = pl.HB; prm.nbands = pl.nbands; prm.halo = pl.halo; prm.SW = pl.SW;
+    prm.div_sw = make_fast_div((unsigned)pl.SW); prm.div_c = make_fast_div((unsigned)g.C); prm.div_nb = make_fast_div((unsigned)pl.nbands);
+    prm.rot = bwd ? 1 : 0; prm.bf16 = bf16 ? 1 : 0;
+    uintptr_t ptrs = reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out);
+    if (mix && !bwd) ptrs |= reinterpret_cast<uintptr_t>(mix->u_out);
+    prm.vec = (g.W % 4 == 0 && (ptrs & (bf16 ? 7 : 15)) == 0) ? 1 : 0;
+    prm.ncw = pl.ncw; prm.niow = pl.niow;
+    prm.bk_warps = pl.bk_warps; prm.bk_parts = pl.bk_parts; prm.bk_per = pl.bk_per; prm.div_bk = make_fast_div((unsigned)pl.bk_warps);
+    prm.off_dummy = pl.off_dummy; prm.off_ring = pl.off_ring; prm.off_a = pl.off_a; prm.off_w = pl.off_w; prm.off_li = pl.off_li;
+    if (mix) {
+        prm.mix_V = mix->V; prm.mix_s = mix->s; prm.mix_b = mix->b;
+        prm.mix_out = bwd ? nullptr : mix->u_out;
+        prm.mix_in = (bwd && mix->grad_in) ? 1 : 0;
+    }
+    prm.logdet_out = bwd ? nullptr : logdet_out;
+    const bool dep = opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0;
+    switch (g.k) {
+    case 2: return invconv_internal::launch_line_k2(pl, prm, dep, st);
+    case 3: return invconv_internal::launch_line_k3(pl, prm, dep, st);
+    case 5: return invconv_internal::launch_line_k5(pl, prm, dep, st);
+    case 7: return invconv_internal::launch_line_k7(pl, prm, dep, st);
+    case 9: return invconv_internal::launch_line_k9(pl, prm, dep, st);
+    case 11: return invconv_internal::launch_line_k11(pl, prm, dep, st);
+    default: return INVCONV_UNSUPPORTED;
+    }
+}
+
 // `bf16`: rhs, out and xsaved are bfloat16 images (see WarpParams::bf16); INVCONV_UNSUPPORTED where the kernel
 // cannot take them (images in global memory, grad_w from the separate kernel, sizes or pointers the bulk copies
 // do not accept) -- the caller then converts around the fp32 path.
@@ -257,6 +230,16 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
                 void* ws, cudaStream_t st, const WarpMix* mix = nullptr, float* logdet_out = nullptr,
                 const LogdetFuse& ld = LogdetFuse{}, bool bf16 = false)
 {
+    if (line_preferred(g.B, g.C, g.H, g.W, g.k) && !(gw && bf16)) {
+        const int rl = launch_line(bwd, rhs, w, out, g, st, mix, logdet_out, bf16);
+        if (rl != INVCONV_UNSUPPORTED) {                // (bfloat16 images of several bands stay with the warp kernel)
+            if (rl || !gw) return rl;
+            const GradWSmallPlan gs = gradw_small_plan(g.B, g.C, g.H, g.W, g.k);
+            if (ws && gs.ok) return launch_gradw_small(gs, out, xsaved, gw, g, ws, st, ld);
+            generic_grad_w_kernel<<<g.C * g.C * g.k * g.k, 128, 0, st>>>(out, xsaved, gw, g, ld);
+            return check_launch();
+        }
+    }
     const WarpPlan pl = plan_warp(g.B, g.C, g.H, g.W, g.k, bwd);
     if (!pl.ok) return INVCONV_UNSUPPORTED;
     if (mix && pl.glb) return INVCONV_UNSUPPORTED;       // images in global memory: the caller composes the step
@@ -285,12 +268,15 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
     }
     prm.glb = pl.glb ? 1 : 0;
     prm.vec = (aligned && g.W % 4 == 0) ? 1 : 0;
+    const bool ring = opt(INVCONV_OPT_WARP_RING) != 0, split = opt(INVCONV_OPT_WARP_CHANNEL_SPLIT) != 0, dep = opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0;
     int rc = INVCONV_UNSUPPORTED;
-#define X(CC, KK)                                                                         \
-    if (g.C == CC && g.k == KK)                                                           \
-        rc = bwd ? launch_warp_ck<CC, KK, true>(pl, prm, st) : launch_warp_ck<CC, KK, false>(pl, prm, st);
-    INVCONV_WARP_CASES(X)
-#undef X
+    switch (g.C) {
+    case 1: rc = invconv_internal::launch_warp_c1(g.k, bwd, pl, prm, ring, split, dep, st); break;
+    case 2: rc = invconv_internal::launch_warp_c2(g.k, bwd, pl, prm, ring, split, dep, st); break;
+    case 3: rc = invconv_internal::launch_warp_c3(g.k, bwd, pl, prm, ring, split, dep, st); break;
+    case 4: rc = invconv_internal::launch_warp_c4(g.k, bwd, pl, prm, ring, split, dep, st); break;
+    default: break;
+    }
     if (rc || !separate) return rc;
     return launch_gradw_small(gs, out, xsaved, gw, g, ws, st, ld);
 }
@@ -307,63 +293,6 @@ size_t warp_workspace_bytes(int B, int C, int H, int W, int k)
 }
 
 // ---------------------------------------------------------------- masked convolution, few channels
-template <int C, int K>
-int launch_masked_conv_ck(const float* x, const float* w, float* y, Geom g, cudaStream_t st)
-{
-    // warps per band of rows: one, or one per output channel where the kernel does not fit a lane's registers
-    constexpr int wsplit = (C * C * K * K <= 108) ? 1 : C;
-    constexpr int maxw = 8 / wsplit;             // eight warps per CTA
-    int wpi = (g.H + 7) / 8;                     // about eight rows per warp
-    if (wpi > maxw) wpi = maxw;
-    if (wpi < 1) wpi = 1;
-    int ipc = maxw / wpi;
-    if (ipc > g.B) ipc = g.B;
-    if (ipc < 1) ipc = 1;
-    while (ipc > 1 && masked_conv_smem<C, K>(g.H, g.W, ipc) > kMaxDynSmem) --ipc;
-    size_t smem = masked_conv_smem<C, K>(g.H, g.W, ipc);
-    const size_t chw = (size_t)g.C * g.H * g.W;
-    ConvParams prm;
-    prm.x = x; prm.w = w; prm.y = y; prm.B = g.B; prm.H = g.H; prm.W = g.W;
-    prm.bulk = ((reinterpret_cast<uintptr_t>(x) & 15) == 0 && chw % 4 == 0) ? 1 : 0;
-    int grid = (g.B + ipc - 1) / ipc;
-    // few (fewer CTAs than half the SMs) or very large images: one CTA per band of rows instead, about two CTAs per SM
-    const bool rows_ok = (reinterpret_cast<uintptr_t>(x) & 15) == 0 && g.W % 4 == 0;
-    if (rows_ok && g.H >= 16 && (smem > kMaxDynSmem || 2 * grid <= sm_count())) {
-        int bands = (2 * sm_count() + g.B - 1) / g.B;
-        if (bands > (g.H + 7) / 8) bands = (g.H + 7) / 8;             // at least eight rows per band
-        int bh = (g.H + bands - 1) / bands;
-        while (masked_conv_smem<C, K>(bh + K - 1, g.W, 1) > kMaxDynSmem && bh > 1) bh = (bh + 1) / 2;
-        bands = (g.H + bh - 1) / bh;
-        if (bands > 1 && masked_conv_smem<C, K>(bh + K - 1, g.W, 1) <= kMaxDynSmem) {
-            prm.bands = bands; prm.bh = bh; prm.bulk = 1;
-            ipc = 1;
-            wpi = bh >= 16 ? 4 : (bh >= 8 ? 2 : 1);
-            if (wpi > maxw) wpi = maxw;
-            smem = masked_conv_smem<C, K>(bh + K - 1, g.W, 1);
-            grid = g.B * bands;
-        }
-    }
-    if (smem > kMaxDynSmem) return INVCONV_UNSUPPORTED;
-    auto kern = masked_conv_warp_kernel<C, K>;
-    const int rc = set_smem_limit(kern, smem);
-    if (rc) return rc;
-    prm.ipc = ipc; prm.wpi = wpi;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(ipc * wpi * wsplit * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // launch latency overlaps the kernel before
-    attr[0].val.programmaticStreamSerializationAllowed = opt(INVCONV_OPT_DEPENDENT_LAUNCH) ? 1 : 0;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, prm) != cudaSuccess) {
-        cudaGetLastError();
-        return INVCONV_CUDA_ERROR;
-    }
-    return check_launch();
-}
-
 template <int K>
 int launch_masked_conv_tile_k(const ConvTilePlan& pl, const ConvTileParams& prm, cudaStream_t st)
 {
@@ -400,10 +329,14 @@ int launch_masked_conv_tile(const float* x, const float* w, float* y, Geom g, cu
 
 int launch_masked_conv_small(const float* x, const float* w, float* y, Geom g, cudaStream_t st)
 {
-#define X(CC, KK) if (g.C == CC && g.k == KK) return launch_masked_conv_ck<CC, KK>(x, w, y, g, st);
-    INVCONV_WARP_CASES(X)
-#undef X
-    return INVCONV_UNSUPPORTED;
+    const bool dep = opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0;
+    switch (g.C) {
+    case 1: return invconv_internal::launch_masked_conv_c1(x, w, y, g, dep, st);
+    case 2: return invconv_internal::launch_masked_conv_c2(x, w, y, g, dep, st);
+    case 3: return invconv_internal::launch_masked_conv_c3(x, w, y, g, dep, st);
+    case 4: return invconv_internal::launch_masked_conv_c4(x, w, y, g, dep, st);
+    default: return INVCONV_UNSUPPORTED;
+    }
 }
 
 // ---------------------------------------------------------------- team family
@@ -478,11 +411,17 @@ GradWTensorPlan gradw_tensor_plan(int B, int C, int H, int W, int k)
     return plan_gradw_tensor(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count());
 }
 
+// The team family: a cluster or CTA per image (team_kernels.cuh), or the line wavefront where that has a plan.
+bool team_serves(int B, int C, int H, int W, int k)
+{
+    return team_plan(B, C, H, W, k).ok || line_plan(B > 0 ? B : 1, C, H, W, k).ok;
+}
+
 // Workspace of the team family: control words, transformed kernel, C*C floats, then the partial sums of
 // grad_w -- one set per batch share of whichever correlation kernel runs (the tcgen05 one included).
 size_t team_workspace_bytes(int B, int C, int H, int W, int k)
 {
-    if (!team_plan(B, C, H, W, k).ok) return 0;
+    if (!team_serves(B, C, H, W, k)) return 0;
     const size_t na = sizeof(float) * (size_t)k * k * C * C;
     const GradWPlan gp = gradw_plan(B, C, H, W, k);
     const GradWTensorPlan gt = gradw_tensor_plan(B, C, H, W, k);
@@ -622,6 +561,11 @@ int launch_pixel_inst(const TeamPlan& pl, const TeamParams& prm, cudaStream_t st
 int launch_team(bool bwd, const float* rhs, const float* w, float* out, Geom g, void* ws, cudaStream_t st, float* logdet_out = nullptr)
 {
     const TeamPlan pl = team_plan(g.B, g.C, g.H, g.W, g.k);
+    const bool variant = opt(INVCONV_OPT_TEAM_VARIANT) == 1 || opt(INVCONV_OPT_TEAM_VARIANT) == 2;
+    if ((!pl.ok && !variant) || line_preferred(g.B, g.C, g.H, g.W, g.k)) {
+        const int rl = launch_line(bwd, rhs, w, out, g, st, nullptr, logdet_out);
+        if (rl != INVCONV_UNSUPPORTED) return rl;
+    }
     if (!pl.ok) return INVCONV_UNSUPPORTED;
     float* A = reinterpret_cast<float*>(static_cast<char*>(ws) + INVCONV_WS_CONTROL_BYTES);
     {
@@ -727,8 +671,37 @@ int auto_path(int B, int C, int H, int W, int k)
 {
     if (plan_warp(B > 0 ? B : 1, C, H, W, k, true).ok) return INVCONV_PATH_WARP;
     if (tensor_plan(B, C, H, W, k).ok) return INVCONV_PATH_TENSOR;
-    if (team_plan(B, C, H, W, k).ok) return INVCONV_PATH_TEAM;
+    if (team_serves(B, C, H, W, k)) return INVCONV_PATH_TEAM;
     return INVCONV_PATH_GENERIC;
+}
+
+// Whether the line wavefront runs in place of the family that the shape belongs to (INVCONV_OPT_LINE overrides; a forced family
+// runs its own kernels).
+bool line_preferred(int B, int C, int H, int W, int k)
+{
+    const int knob = opt(INVCONV_OPT_LINE);
+    if (knob == 0 || B < 1) return false;
+    const LinePlan pl = line_plan(B, C, H, W, k);
+    if (!pl.ok) return false;
+    if (knob == 1) return true;
+    if (g_forced_path.load() != INVCONV_PATH_AUTO) return false;
+    const WarpPlan wp = plan_warp(B, C, H, W, k, true);
+    if (!wp.ok) {
+        // TENSOR and TEAM shapes: measured (16x16, k = 3, batch 64) 14.5 against 38 us at C = 12, 16.5 against 43 us at C = 16, but
+        // 95 against 60 us at C = 24, where a CTA's registers no longer hold a band of useful height
+        return C <= 16;
+    }
+    // WARP shapes.  One lane per row keeps its taps in registers and needs no barrier: it wins while they fit (few channels, k up to
+    // 3) and one warp covers the rows.  Measured, us (WARP / line): C = 3, k = 3: 10.6 / 11.8 at 32x32, 27.8 / 22.0 at 64x64
+    // (batch 32; 28.6 / 31.7 at batch 256), 244 / 215 at 256x256; C = 3, k = 5: 31 / 13 at 32x32; C = 4, k = 3: 13.5 / 12.0 at
+    // 32x32 (14.0 / 17.3 at batch 256); C = 2, k = 5: 10.6 / 11.8 at 32x32, 34.6 / 20.7 at 64x64; C = 1: WARP throughout
+    if (C == 1) return false;
+    if (k == 5) return C >= 3 || H > 32;
+    if (wp.glb) return true;
+    const bool few = B <= sm_count();              // one image per SM: latency counts, not throughput
+    if (C == 2) return H > 32 && W % 4 != 0;
+    if (C == 3) return H > 32 && few;
+    return few && (H > 32 || k == 3);
 }
 
 int resolve_path(int B, int C, int H, int W, int k)
@@ -771,8 +744,9 @@ int launch_forward(int path, const float* y, const float* w, float* x, Geom g,
         // buffers off a 16-byte boundary cannot use the bulk copies of the tensor family: the team family serves
         // them from the same workspace (its layout is a prefix of the tensor family's)
         const bool aligned = ((reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
+        if (line_preferred(g.B, g.C, g.H, g.W, g.k)) return launch_team(false, y, w, x, g, ws, st, logdet_out);
         if (!aligned && g_forced_path.load() == INVCONV_PATH_AUTO) {
-            if (team_plan(g.B, g.C, g.H, g.W, g.k).ok) return launch_team(false, y, w, x, g, ws, st, logdet_out);
+            if (team_serves(g.B, g.C, g.H, g.W, g.k)) return launch_team(false, y, w, x, g, ws, st, logdet_out);
             generic_wavefront_kernel<false><<<g.B, 256, 0, st>>>(y, w, x, g);      // neither family takes them: the generic one does
             const int rc = check_launch();
             return rc ? rc : separate_logdet();
@@ -821,8 +795,10 @@ int launch_backward(int path, const float* gx, const float* x, const float* w, f
         if (g.B > 0) {
             const bool aligned = ((reinterpret_cast<uintptr_t>(gx) | reinterpret_cast<uintptr_t>(gy)) & 15) == 0;
             int rc;
-            if (!aligned && g_forced_path.load() == INVCONV_PATH_AUTO) {
-                if (team_plan(g.B, g.C, g.H, g.W, g.k).ok) {
+            if (line_preferred(g.B, g.C, g.H, g.W, g.k)) {
+                rc = launch_team(true, gx, w, gy, g, ws, st);
+            } else if (!aligned && g_forced_path.load() == INVCONV_PATH_AUTO) {
+                if (team_serves(g.B, g.C, g.H, g.W, g.k)) {
                     rc = launch_team(true, gx, w, gy, g, ws, st);
                 } else {
                     generic_wavefront_kernel<true><<<g.B, 256, 0, st>>>(gx, w, gy, g);
@@ -1079,6 +1055,10 @@ int invconv_forward_bf16_ws(const void* y, const float* w, void* x, int B, int C
                                    nullptr, nullptr, LogdetFuse{}, true);
         if (rw != INVCONV_UNSUPPORTED) return rw;
     }
+    if (path != INVCONV_PATH_WARP && line_preferred(B, C, H, W, k)) {
+        const int rl = launch_line(false, y, w, x, g, st, nullptr, nullptr, true);
+        if (rl != INVCONV_UNSUPPORTED) return rl;
+    }
     const size_t n = (size_t)B * C * H * W, act = up256(n * sizeof(float));
     if (workspace_bytes < need + 2 * act) return INVCONV_WORKSPACE_TOO_SMALL;
     float* y32 = reinterpret_cast<float*>(static_cast<char*>(workspace) + need);
@@ -1112,6 +1092,10 @@ int invconv_backward_bf16_ws(const void* grad_x, const void* x, const float* w, 
         const int rw = launch_warp(true, static_cast<const float*>(grad_x), w, static_cast<float*>(grad_y),
                                    static_cast<const float*>(x), grad_w, g, workspace, st, nullptr, nullptr, LogdetFuse{}, true);
         if (rw != INVCONV_UNSUPPORTED) return rw;
+    }
+    if (path != INVCONV_PATH_WARP && !grad_w && line_preferred(B, C, H, W, k)) {
+        const int rl = launch_line(true, grad_x, w, grad_y, g, st, nullptr, nullptr, true);
+        if (rl != INVCONV_UNSUPPORTED) return rl;
     }
     const size_t n = (size_t)B * C * H * W, act = up256(n * sizeof(float));
     if (workspace_bytes < need + 3 * act) return INVCONV_WORKSPACE_TOO_SMALL;

@@ -7,6 +7,15 @@
 
 #include "common.cuh"
 #include "tensor_plan.h"
+#include "line_plan.h"
+#include "warp_plan.h"
+
+namespace invconv {
+struct LineParams;
+struct WarpParams;
+struct GradWSmallPlan;
+struct GradWSmallParams;
+}  // namespace invconv
 
 namespace invconv_internal {
 
@@ -56,5 +65,28 @@ int conv_tensor_launch(const invconv::ConvTensorPlan& pl, const float* x, const 
 // tensor_lib.cu: the tcgen05 correlation kernel of grad_w; partial sums [pl.S][k*k][C][C] go to `partials`.
 int gradw_tensor_launch(const invconv::GradWTensorPlan& pl, const float* gy, const float* x, float* partials,
                         invconv::Geom g, cudaStream_t st);
+
+// warp_c*.cu: the few-channel kernels (WARP family, its grad_w, its masked convolution) of one channel count; INVCONV_UNSUPPORTED
+// for a kernel side they do not have.
+int launch_warp_c1(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
+int launch_gradw_small_c1(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
+int launch_masked_conv_c1(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
+int launch_warp_c2(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
+int launch_gradw_small_c2(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
+int launch_masked_conv_c2(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
+int launch_warp_c3(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
+int launch_gradw_small_c3(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
+int launch_masked_conv_c3(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
+int launch_warp_c4(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
+int launch_gradw_small_c4(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
+int launch_masked_conv_c4(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
+
+// line_k*.cu: the LINE wavefront instances of one kernel side.
+int launch_line_k2(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
+int launch_line_k3(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
+int launch_line_k5(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
+int launch_line_k7(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
+int launch_line_k9(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
+int launch_line_k11(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);
 
 }  // namespace invconv_internal
