@@ -1,249 +1,11 @@
-// Weight gradient for wide channel counts (Theorem 2 in closed form):
-//   grad_w[co][ci][K-1-dh][K-1-dw] = - sum_{n,h,w} grad_y[n,co,h,w] * x[n,ci,h-dh,w-dw]
-// This is a correlation with contraction length B*H*W -- a batched reduction
-// with C*C*K*K outputs, bound by the fp32 FMA pipe.
-//
-// Output-stationary tiling: a CTA owns one kernel row dh, a 16*TC x 16*TC tile
-// of (co, ci) pairs and a share of the batch; thread (tc, ti) keeps the
-// TC x TC x K partial sums of its channel pairs in registers.  For every image
-// of its share the CTA stages the tile's grad_y and x channel planes in shared
-// memory with bulk (TMA) copies -- channel planes are contiguous in NCHW -- and
-// walks the rows in quads of four pixels: one 16-byte load per grad_y channel,
-// two per x channel (the K-1 columns to the left come with the aligned quad
-// before), 4*TC*TC*K FMAs.  The channel planes are padded in shared memory so
-// that the 16 threads that differ in ci hit disjoint banks.
-// Batch shares write partial sums; gradw_reduce_kernel adds them in a fixed
-// order, negates and applies the channel mask.
+// Weight gradient: the sum over the shares of a correlation kernel (gradw_quad.cuh, gradw_tensor.cuh), and the correlation of
+// the few-channel family.
 #pragma once
 
 #include "common.cuh"
 #include "tma.cuh"
 
 namespace invconv {
-
-struct GradWParams {
-    const float* gy;       // [B][C][H][W]
-    const float* x;        // [B][C][H][W]
-    float* partials;       // [nbc][K*K][C][C]   (tap = dh*K + dw, then co, then ci)
-    int B, C, H, W;
-    int nbc;               // batch shares
-    int tiles;             // channel tiles per side
-    int plane;             // floats per channel plane in shared memory (H*W + padding)
-};
-
-template <int TC, int K>
-__global__ void __launch_bounds__(256) gradw_tile_kernel(GradWParams p)
-{
-    extern __shared__ __align__(128) float smem[];
-    __shared__ unsigned long long bar;
-    constexpr int TB = 16 * TC;                 // channels per tile side
-    const int H = p.H, W = p.W, HW = H * W, C = p.C;
-    const int tid = threadIdx.x;
-    const int tc = tid >> 4, ti = tid & 15;
-    int bid = blockIdx.x;
-    const int share = bid % p.nbc; bid /= p.nbc;
-    const int tci = bid % p.tiles; bid /= p.tiles;
-    const int tco = bid % p.tiles; bid /= p.tiles;
-    const int dh = bid;
-    const int co0 = tco * TB, ci0 = tci * TB;
-    const int nco = min(TB, C - co0), nci = min(TB, C - ci0);
-    float* gys = smem;                          // [TB][plane]
-    float* xs = smem + TB * p.plane;            // [TB][plane]
-
-    float acc[TC][TC][K];
-#pragma unroll
-    for (int i = 0; i < TC; ++i)
-#pragma unroll
-        for (int j = 0; j < TC; ++j)
-#pragma unroll
-            for (int d = 0; d < K; ++d) acc[i][j][d] = 0.f;
-
-    if (tid == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
-    for (int i = tid; i < 2 * TB * p.plane; i += blockDim.x) smem[i] = 0.f;   // channels beyond C stay zero
-    __syncthreads();
-
-    unsigned phase = 0;
-    bool ok = true;
-    for (int n = share; n < p.B; n += p.nbc) {
-        if (tid < 32) {
-            // one warp issues the per-channel bulk copies of this image's two tiles
-            fence_proxy_async();
-            if (tid == 0) mbar_expect_tx(&bar, (unsigned)((nco + nci) * HW * 4));
-            __syncwarp();
-            const float* gsrc = p.gy + ((size_t)n * C + co0) * HW;
-            const float* xsrc = p.x + ((size_t)n * C + ci0) * HW;
-            for (int c = tid; c < nco; c += 32) bulk_g2s(gys + c * p.plane, gsrc + (size_t)c * HW, (unsigned)HW * 4u, &bar);
-            for (int c = tid; c < nci; c += 32) bulk_g2s(xs + c * p.plane, xsrc + (size_t)c * HW, (unsigned)HW * 4u, &bar);
-        }
-        ok = mbar_wait_bounded(&bar, phase);
-        phase ^= 1u;
-        if (!__syncthreads_and(ok)) { if (tid == 0) raise_status(INVCONV_TIMEOUT); break; }
-
-        const float* gq[TC];
-        const float* xq[TC];
-#pragma unroll
-        for (int i = 0; i < TC; ++i) gq[i] = gys + (tc * TC + i) * p.plane;
-#pragma unroll
-        for (int j = 0; j < TC; ++j) xq[j] = xs + (ti * TC + j) * p.plane;
-        for (int h = dh; h < H; ++h) {
-            for (int w0 = 0; w0 < W; w0 += 4) {
-                float g[TC][4], v[TC][8];
-#pragma unroll
-                for (int i = 0; i < TC; ++i) {
-                    const float4 t = *reinterpret_cast<const float4*>(gq[i] + h * W + w0);
-                    g[i][0] = t.x; g[i][1] = t.y; g[i][2] = t.z; g[i][3] = t.w;
-                }
-#pragma unroll
-                for (int j = 0; j < TC; ++j) {
-                    const float* row = xq[j] + (h - dh) * W + w0;
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (K > 1 && w0 > 0) a = *reinterpret_cast<const float4*>(row - 4);
-                    const float4 b = *reinterpret_cast<const float4*>(row);
-                    v[j][0] = a.x; v[j][1] = a.y; v[j][2] = a.z; v[j][3] = a.w;
-                    v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
-                }
-#pragma unroll
-                for (int d = 0; d < K; ++d)
-#pragma unroll
-                    for (int px = 0; px < 4; ++px)
-#pragma unroll
-                        for (int i = 0; i < TC; ++i)
-#pragma unroll
-                            for (int j = 0; j < TC; ++j)
-                                acc[i][j][d] = fmaf(g[i][px], v[j][4 + px - d], acc[i][j][d]);
-            }
-        }
-        __syncthreads();       // everyone is done with this image before its planes are overwritten
-    }
-
-    float* dst = p.partials + (size_t)share * K * K * C * C;
-#pragma unroll
-    for (int i = 0; i < TC; ++i)
-#pragma unroll
-        for (int j = 0; j < TC; ++j) {
-            const int co = co0 + tc * TC + i, ci = ci0 + ti * TC + j;
-            if (co < C && ci < C) {
-#pragma unroll
-                for (int d = 0; d < K; ++d) dst[((size_t)(dh * K + d) * C + co) * C + ci] = acc[i][j][d];
-            }
-        }
-}
-
-// ---------------------------------------------------------------------------
-// The same tiling on the tensor pipe (TF32 inputs, fp32 accumulation): for a
-// fixed tap the sum over pixels is a matrix product  G[co][ci] = sum_p
-// grad_y[co][p] * x[ci][p - shift], M = co, N = ci, contraction over the
-// pixels, which are the contiguous index of both operands in NCHW.  A warp
-// owns one 16-row block of output channels and one kernel column dw and walks
-// the rows h >= dh of the staged planes in chunks of eight pixels:
-// mma.m16n8k8 with A = grad_y[16 co][8 pixels], B = x[8 pixels - shift][8 ci]
-// for each of the tile's 8-channel groups.  Fragments are read straight from
-// the padded channel planes (plane stride = 4 mod 32: the 8 x 4 elements of a
-// fragment register fall in 32 different banks); the K-1 pixels to the left of
-// column 0 and the rows above row 0 are zeros by predicate.  Inputs are
-// rounded to TF32 (10-bit mantissa): the weight gradient's parity bar is 1e-3
-// of its largest entry, which a single TF32 pass holds (the solves, at 1e-4,
-// stay in fp32).  Needs W % 8 == 0; other shapes use the FMA kernel above.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned to_tf32(float v)
-{
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
-    return r;
-}
-
-__device__ __forceinline__ void mma_tf32_16x8x8(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2])
-{
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// ALLDH (tiles of 16 channels): one CTA covers all K*K taps, warp = (dh, dw), so that a 12- or 16-channel
-// layer still gives every CTA K*K warps and every image is staged once instead of once per kernel row.
-template <int TC, int K, bool ALLDH = false>
-__global__ void __launch_bounds__(32 * (ALLDH ? K * K : TC * K)) gradw_mma_kernel(GradWParams p)
-{
-    static_assert(!ALLDH || TC == 1, "all kernel rows in one CTA: tiles of 16 channels only");
-    extern __shared__ __align__(128) float smem[];
-    constexpr int TB = 16 * TC;                 // channels per tile side
-    constexpr int NT8 = 2 * TC;                 // 8-channel groups of the ci tile
-    const int H = p.H, W = p.W, HW = H * W, C = p.C;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
-    const int g = lane >> 2, t = lane & 3;      // fragment coordinates
-    const int mt = ALLDH ? 0 : warp / K;        // this warp's 16 output channels
-    const int dw = ALLDH ? warp % K : warp - mt * K;   // ... and kernel column
-    int bid = blockIdx.x;
-    const int share = bid % p.nbc; bid /= p.nbc;
-    const int tci = bid % p.tiles; bid /= p.tiles;
-    const int tco = bid % p.tiles; bid /= p.tiles;
-    const int dh = ALLDH ? warp / K : bid;
-    const int co0 = tco * TB, ci0 = tci * TB;
-    const int nco = min(TB, C - co0), nci = min(TB, C - ci0);
-    float* gys = smem;                          // [TB][plane]
-    float* xs = smem + TB * p.plane;            // [TB][plane]
-
-    float acc[NT8][4];
-#pragma unroll
-    for (int i = 0; i < NT8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    // channels beyond C (padding of the last tile) stay zero; the others are overwritten by every image
-    for (int c = nco + warp; c < TB; c += nwarps)
-        for (int i = lane; i < p.plane; i += 32) gys[c * p.plane + i] = 0.f;
-    for (int c = nci + warp; c < TB; c += nwarps)
-        for (int i = lane; i < p.plane; i += 32) xs[c * p.plane + i] = 0.f;
-
-    for (int n = share; n < p.B; n += p.nbc) {
-        // stage the tile's channel planes with 16-byte asynchronous copies issued by all threads (a bulk copy
-        // per channel plane would serialise in the copy engine at ~150 cycles each, more than the whole product)
-        const float* gsrc = p.gy + ((size_t)n * C + co0) * HW;
-        const float* xsrc = p.x + ((size_t)n * C + ci0) * HW;
-        const int nq = HW >> 2;
-        for (int c = warp; c < nco + nci; c += nwarps) {
-            const bool isg = c < nco;
-            const int cc = isg ? c : c - nco;
-            const float* src = (isg ? gsrc : xsrc) + (size_t)cc * HW;
-            float* dstp = (isg ? gys : xs) + cc * p.plane;
-            for (int q = lane; q < nq; q += 32) cp_async_f32x4(dstp + 4 * q, src + 4 * q, true);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-
-        const float* ga = gys + (mt * 16 + g) * p.plane + t;          // A: rows g and g + 8, pixel columns t and t + 4
-        const float* xb = xs + g * p.plane + t - dw;                  // B: channel g of a group, pixels t and t + 4, shifted
-        for (int h = dh; h < H; ++h) {
-            for (int w0 = 0; w0 < W; w0 += 8) {
-                const int pa = h * W + w0, pb = (h - dh) * W + w0;
-                unsigned a[4];
-                a[0] = to_tf32(ga[pa]);
-                a[1] = to_tf32(ga[pa + 8 * p.plane]);
-                a[2] = to_tf32(ga[pa + 4]);
-                a[3] = to_tf32(ga[pa + 8 * p.plane + 4]);
-                const bool v0 = w0 + t >= dw, v1 = w0 + t + 4 >= dw;   // pixels left of column 0 are padding
-#pragma unroll
-                for (int nt = 0; nt < NT8; ++nt) {
-                    unsigned b[2];
-                    b[0] = v0 ? to_tf32(xb[nt * 8 * p.plane + pb]) : 0u;
-                    b[1] = v1 ? to_tf32(xb[nt * 8 * p.plane + pb + 4]) : 0u;
-                    mma_tf32_16x8x8(acc[nt], a, b);
-                }
-            }
-        }
-        __syncthreads();       // everyone is done with this image before its planes are overwritten
-    }
-
-    float* dst = p.partials + (size_t)share * K * K * C * C + (size_t)(dh * K + dw) * C * C;
-#pragma unroll
-    for (int nt = 0; nt < NT8; ++nt)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int co = co0 + mt * 16 + g + (j >> 1) * 8, ci = ci0 + nt * 8 + 2 * t + (j & 1);
-            if (co < C && ci < C) dst[(size_t)co * C + ci] = acc[nt][j];
-        }
-}
 
 // grad_w[co][ci][K-1-dh][K-1-dw] = -(sum over shares), zero outside the channel mask of the centre tap.
 // LANES adjacent lanes share one entry: lane q adds the shares b = q, q+LANES, ... in that order (up to sixteen
@@ -254,6 +16,8 @@ template <int LANES>
 __global__ void __launch_bounds__(256) gradw_reduce_kernel(const float* __restrict__ partials, float* __restrict__ grad_w,
                                                            int nbc, int C, int K, const LogdetFuse ld)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // launched while the correlation still runs
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int EPW = 32 / LANES;                      // entries per warp
     constexpr int INF = LANES == 1 ? 8 : 16;             // loads in flight per thread
     const int NA = K * K * C * C;
@@ -282,52 +46,6 @@ __global__ void __launch_bounds__(256) gradw_reduce_kernel(const float* __restri
             grad_w[((co * C + ci) * K + (K - 1 - dh)) * K + (K - 1 - dw)] = finish_grad_w(s, co, ci, tap, C, K, ld);
         }
     }
-}
-
-struct GradWPlan {
-    bool ok = false;
-    int TC = 3, tiles = 1, nbc = 1, plane = 0, grid = 0;
-    int nbc_all = 0, grid_all = 0;      // tiles of 16 channels on the tensor pipe: shares and CTAs when one CTA covers all taps
-    size_t smem = 0;
-};
-
-inline GradWPlan plan_gradw(int B, int C, int H, int W, int K, size_t max_smem, int sm_count)
-{
-    GradWPlan pl;
-    if (!(K == 1 || K == 2 || K == 3 || K == 5)) return pl;
-    if (W % 4 != 0 || B < 1) return pl;
-    pl.TC = C <= 16 ? 1 : 3;
-    const int TB = 16 * pl.TC;
-    pl.tiles = (C + TB - 1) / TB;
-    const int HW = H * W;
-    int pad = 0;
-    for (; pad < 32; pad += 4) {
-        const int m = (pl.TC * (HW + pad)) % 32;
-        if (m % 8 == 4) break;
-    }
-    if (pad >= 32) pad = 4;
-    pl.plane = HW + pad;
-    pl.smem = sizeof(float) * 2 * (size_t)TB * pl.plane;
-    if (pl.smem > max_smem) return pl;
-    int nbc = (2 * sm_count) / (K * pl.tiles * pl.tiles);
-    if (nbc < 1) nbc = 1;
-    if (nbc > B) nbc = B;
-    // even out the images per share
-    const int per = (B + nbc - 1) / nbc;
-    nbc = (B + per - 1) / per;
-    pl.nbc = nbc;
-    pl.grid = K * pl.tiles * pl.tiles * nbc;
-    if (pl.TC == 1) {
-        int na = (2 * sm_count) / (pl.tiles * pl.tiles);
-        if (na < 1) na = 1;
-        if (na > B) na = B;
-        const int pa = (B + na - 1) / na;
-        na = (B + pa - 1) / pa;
-        pl.nbc_all = na;
-        pl.grid_all = pl.tiles * pl.tiles * na;
-    }
-    pl.ok = true;
-    return pl;
 }
 
 // ---------------------------------------------------------------------------

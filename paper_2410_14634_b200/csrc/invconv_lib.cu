@@ -128,20 +128,21 @@ GradWSmallPlan gradw_small_plan(int B, int C, int H, int W, int k)
     return plan_gradw_small(B, C, H, W, k, kGradWSmallSmem, kMaxDynSmem - 8 * 1024, sm_count());
 }
 
-// Whether grad_w comes from the pixel-parallel kernel after the wavefront instead of riding along in it.
-// Riding along costs every diagonal step C*C*k*k extra multiply-adds on the one warp that owns the rows; the
-// separate kernel costs a launch and a second read of grad_y and x from L2.  Measured on B200, added time of
-// the separate kernel against riding along: 18 us against 10 us (C=3, 32x32, k=3, batch 128), 11 us against
-// 4 us (C=1, 28x28, k=3, batch 256), 13 us against 118 us (C=3, 64x64, k=5, batch 16, where the sums do not
-// fit the wavefront's registers), 24 us against 75 us (C=1, 256x256, k=5, batch 4, images in global memory).
-// So it is used where the sums do not fit the registers or the images stay in global memory (INVCONV_OPT_GRADW_SEPARATE overrides).
-bool gradw_separate(const WarpPlan& pl, const GradWSmallPlan& gs, int C, int k)
+// Whether grad_w comes from a correlation kernel after the wavefront instead of riding along in it.
+// Riding along costs every diagonal step C*C*k*k extra multiply-adds on the one warp that owns the rows; the separate kernel costs
+// two launches and a second read of grad_y and x from L2.  Measured on B200, added time of the separate kernel against
+// riding along: 13 us against 11 us (C=3, 32x32, k=3, batch 256), 10 us against 4 us (C=1, 28x28, k=3, batch 256), 8 us
+// against 118 us (C=3, 64x64, k=5, batch 16, where the sums do not fit the wavefront's registers), 9 us against 75 us (C=1,
+// 256x256, k=5, batch 4, images in global memory), 6 us against 10 us (C=3, 64x64, k=3, one image: several row blocks wait
+// for one another).  bfloat16 images are converted in the wavefront kernel only while grad_w rides along, so they keep it.
+// INVCONV_OPT_GRADW_SEPARATE overrides.
+bool gradw_separate(const WarpPlan& pl, const GradWSmallPlan& gs, int C, int H, int k, bool bf16)
 {
     if (!gs.ok) return false;
     const int knob = opt(INVCONV_OPT_GRADW_SEPARATE);
     if (knob == 0) return false;
     if (knob == 1) return true;
-    return pl.glb || C * C * k * k > 81;
+    return pl.glb || C * C * k * k > 81 || (!bf16 && C >= 3 && H > 32);
 }
 
 int launch_gradw_small(const GradWSmallPlan& gs, const float* gy, const float* x, float* gw, Geom g, void* ws, cudaStream_t st,
@@ -162,13 +163,57 @@ int launch_gradw_small(const GradWSmallPlan& gs, const float* gy, const float* x
     prm.div_xr = make_fast_div((unsigned)(gs.RB + g.k - 1));
     prm.div_qpr = make_fast_div((unsigned)(gs.gst / 4));
     const bool dep = opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0;
-    switch (g.C) {
-    case 1: return invconv_internal::launch_gradw_small_c1(g.k, gs, prm, dep, st);
-    case 2: return invconv_internal::launch_gradw_small_c2(g.k, gs, prm, dep, st);
-    case 3: return invconv_internal::launch_gradw_small_c3(g.k, gs, prm, dep, st);
-    case 4: return invconv_internal::launch_gradw_small_c4(g.k, gs, prm, dep, st);
-    default: return INVCONV_UNSUPPORTED;
+    return invconv_internal::launch_gradw_small_c1(g.k, gs, prm, dep, st);
+}
+
+GradWQuadPlan gradw_quad_plan(int B, int C, int H, int W, int k)
+{
+    return plan_gradw_quad(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count());
+}
+
+// Fixed-order sum of the shares' partial sums into grad_w.
+int launch_gradw_reduce(const float* partials, float* gw, int shares, Geom g, cudaStream_t st, const LogdetFuse& ld)
+{
+    const size_t na = (size_t)g.k * g.k * g.C * g.C;
+    const bool few = na < 16384;        // few entries: four lanes per entry (64 entries per CTA)
+    auto kern = few ? gradw_reduce_kernel<4> : gradw_reduce_kernel<1>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(few ? (na + 63) / 64 : std::min<size_t>((na + 255) / 256, 4096)));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = opt(INVCONV_OPT_DEPENDENT_LAUNCH) ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, partials, gw, shares, g.C, g.k, ld) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
+    return check_launch();
+}
+
+// grad_w through the fp32 correlation kernel (gradw_quad.cuh); `partials`: [shares][k*k][C][C] floats of scratch.
+int launch_gradw_quad(const float* gy, const float* x, float* gw, Geom g, float* partials, cudaStream_t st, const LogdetFuse& ld)
+{
+    const GradWQuadPlan gq = gradw_quad_plan(g.B, g.C, g.H, g.W, g.k);
+    if (!gq.ok || g.B == 0) {
+        generic_grad_w_kernel<<<g.C * g.C * g.k * g.k, 128, 0, st>>>(gy, x, gw, g, ld);
+        return check_launch();
     }
+    const int rc = invconv_internal::gradw_quad_launch(gq, gy, x, partials, g, opt(INVCONV_OPT_DEPENDENT_LAUNCH) != 0, st);
+    return rc ? rc : launch_gradw_reduce(partials, gw, gq.shares, g, st, ld);
+}
+
+// grad_w of the few-channel family after the wavefront: one channel leaves the tiles of the general kernel nothing to share
+// (9.3 against 7.3 us at 4x1x256x256, k = 5); from two on it is the faster one (8.9 against 17.8 us at 64x3x32x32, k = 5).
+int launch_gradw_few(const GradWSmallPlan& gs, const float* gy, const float* x, float* gw, Geom g, void* ws, cudaStream_t st,
+                     const LogdetFuse& ld)
+{
+    if (g.C == 1 && gs.ok) return launch_gradw_small(gs, gy, x, gw, g, ws, st, ld);
+    return launch_gradw_quad(gy, x, gw, g, reinterpret_cast<float*>(static_cast<char*>(ws) + INVCONV_WS_CONTROL_BYTES), st, ld);
+}
+
+size_t gradw_quad_floats(int B, int C, int H, int W, int k)
+{
+    const GradWQuadPlan gq = gradw_quad_plan(B, C, H, W, k);
+    return gq.ok ? (size_t)gq.shares * k * k * C * C : 0;
 }
 
 // The per-pixel neighbours of the layer in a flow step, applied inside the wavefront kernel (see WarpParams).
@@ -235,16 +280,14 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
         if (rl != INVCONV_UNSUPPORTED) {                // (bfloat16 images of several bands stay with the warp kernel)
             if (rl || !gw) return rl;
             const GradWSmallPlan gs = gradw_small_plan(g.B, g.C, g.H, g.W, g.k);
-            if (ws && gs.ok) return launch_gradw_small(gs, out, xsaved, gw, g, ws, st, ld);
-            generic_grad_w_kernel<<<g.C * g.C * g.k * g.k, 128, 0, st>>>(out, xsaved, gw, g, ld);
-            return check_launch();
+            return launch_gradw_few(gs, static_cast<const float*>(out), xsaved, gw, g, ws, st, ld);
         }
     }
     const WarpPlan pl = plan_warp(g.B, g.C, g.H, g.W, g.k, bwd);
     if (!pl.ok) return INVCONV_UNSUPPORTED;
     if (mix && pl.glb) return INVCONV_UNSUPPORTED;       // images in global memory: the caller composes the step
     const GradWSmallPlan gs = (bwd && gw) ? gradw_small_plan(g.B, g.C, g.H, g.W, g.k) : GradWSmallPlan{};
-    const bool separate = bwd && gw && ws && gradw_separate(pl, gs, g.C, g.k);
+    const bool separate = bwd && gw && ws && gradw_separate(pl, gs, g.C, g.H, g.k, bf16);
     if (bf16 && (pl.glb || separate || mix)) return INVCONV_UNSUPPORTED;
     WarpParams prm;
     prm.rhs = rhs; prm.w = w; prm.out = out; prm.xsaved = xsaved; prm.grad_w = separate ? nullptr : gw;
@@ -278,7 +321,7 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
     default: break;
     }
     if (rc || !separate) return rc;
-    return launch_gradw_small(gs, out, xsaved, gw, g, ws, st, ld);
+    return launch_gradw_few(gs, out, xsaved, gw, g, ws, st, ld);
 }
 
 size_t warp_workspace_bytes(int B, int C, int H, int W, int k)
@@ -289,6 +332,7 @@ size_t warp_workspace_bytes(int B, int C, int H, int W, int k)
     size_t floats = (size_t)pl.grid * na;
     const GradWSmallPlan gs = gradw_small_plan(B > 0 ? B : 1, C, H, W, k);
     if (gs.ok && (size_t)gs.grid * ((na + 3) & ~(size_t)3) > floats) floats = (size_t)gs.grid * ((na + 3) & ~(size_t)3);
+    floats = std::max(floats, gradw_quad_floats(B > 0 ? B : 1, C, H, W, k));
     return INVCONV_WS_CONTROL_BYTES + sizeof(float) * floats;
 }
 
@@ -401,11 +445,6 @@ TeamPlan team_plan(int B, int C, int H, int W, int k)
     return plan_team(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count(), opt(INVCONV_OPT_TEAM_VARIANT), opt(INVCONV_OPT_TEAM_CLUSTER));
 }
 
-GradWPlan gradw_plan(int B, int C, int H, int W, int k)
-{
-    return plan_gradw(B, C, H, W, k, kMaxDynSmem / 2, sm_count());      // two CTAs per SM
-}
-
 GradWTensorPlan gradw_tensor_plan(int B, int C, int H, int W, int k)
 {
     return plan_gradw_tensor(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count());
@@ -423,86 +462,18 @@ size_t team_workspace_bytes(int B, int C, int H, int W, int k)
 {
     if (!team_serves(B, C, H, W, k)) return 0;
     const size_t na = sizeof(float) * (size_t)k * k * C * C;
-    const GradWPlan gp = gradw_plan(B, C, H, W, k);
     const GradWTensorPlan gt = gradw_tensor_plan(B, C, H, W, k);
-    int shares = gp.ok ? (gp.nbc > gp.nbc_all ? gp.nbc : gp.nbc_all) : 0;
+    int shares = gradw_quad_plan(B, C, H, W, k).shares;
     if (gt.ok && gt.S > shares) shares = gt.S;
     return INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)C * C + na * shares;
 }
 
-template <int TC, int K>
-int launch_gradw_inst(const GradWPlan& gp, const GradWParams& prm, cudaStream_t st)
-{
-    auto kern = gradw_tile_kernel<TC, K>;
-    const int rc = set_smem_limit(kern, gp.smem);
-    if (rc) return rc;
-    kern<<<gp.grid, 256, gp.smem, st>>>(prm);
-    return check_launch();
-}
-
-template <int TC, int K>
-int launch_gradw_mma_inst(const GradWPlan& gp, const GradWParams& prm, cudaStream_t st)
-{
-    auto kern = gradw_mma_kernel<TC, K>;
-    const int rc = set_smem_limit(kern, gp.smem);
-    if (rc) return rc;
-    kern<<<gp.grid, 32 * TC * K, gp.smem, st>>>(prm);
-    return check_launch();
-}
-
-template <int K>
-int launch_gradw_mma_all_inst(const GradWPlan& gp, const GradWParams& prm, cudaStream_t st)
-{
-    auto kern = gradw_mma_kernel<1, K, true>;
-    const int rc = set_smem_limit(kern, gp.smem);
-    if (rc) return rc;
-    kern<<<gp.grid_all, 32 * K * K, gp.smem, st>>>(prm);
-    return check_launch();
-}
-
-// grad_w through the tiled correlation kernel; partial sums live behind the transformed kernel in the workspace.
+// grad_w in fp32; the partial sums live behind the transformed kernel in the workspace.
 int launch_gradw(const float* gy, const float* x, float* gw, Geom g, void* ws, cudaStream_t st, const LogdetFuse& ld)
 {
-    const GradWPlan gp = gradw_plan(g.B, g.C, g.H, g.W, g.k);
-    const bool aligned = ((reinterpret_cast<uintptr_t>(gy) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
-    if (!gp.ok || !aligned || g.B == 0) {
-        generic_grad_w_kernel<<<g.C * g.C * g.k * g.k, 128, 0, st>>>(gy, x, gw, g, ld);
-        return check_launch();
-    }
     const size_t na = (size_t)g.k * g.k * g.C * g.C;
-    GradWParams prm;
-    prm.gy = gy; prm.x = x;
-    prm.partials = reinterpret_cast<float*>(static_cast<char*>(ws) + INVCONV_WS_CONTROL_BYTES) + na + (size_t)g.C * g.C;
-    prm.B = g.B; prm.C = g.C; prm.H = g.H; prm.W = g.W; prm.nbc = gp.nbc; prm.tiles = gp.tiles; prm.plane = gp.plane;
-    int rc = INVCONV_UNSUPPORTED;
-    // tensor pipe (TF32 inputs) where the fragments line up: rows of whole 8-pixel chunks, conflict-free planes
-    // (measured, kernel + reduction: 31 / 58 us against 41 / 87 us for the FMA kernel on the 48-channel shapes,
-    // k = 3 / 5; 19 us against 25 us on the 12-channel one with all taps in one CTA)
-    // Not below 8 channels: with a handful of entries none of them is large against the cancellation in its own sum,
-    // and TF32 rounding (2^-11 per operand) then shows at 1e-3 of the entry (seen at C = 1, 2 with k = 1).
-    const bool mma = g.C >= 8 && g.W % 8 == 0 && gp.plane % 32 == 4 && opt(INVCONV_OPT_GRADW_TENSOR_PIPE) != 0;
-    int shares = gp.nbc;
-    if (mma && gp.TC == 1) {                 // tiles of 16 channels: one CTA covers all taps, its own share count
-        shares = gp.nbc_all;
-        prm.nbc = shares;
-        if (g.k == 1) rc = launch_gradw_mma_all_inst<1>(gp, prm, st);
-        if (g.k == 2) rc = launch_gradw_mma_all_inst<2>(gp, prm, st);
-        if (g.k == 3) rc = launch_gradw_mma_all_inst<3>(gp, prm, st);
-        if (g.k == 5) rc = launch_gradw_mma_all_inst<5>(gp, prm, st);
-    } else {
-#define X(TT, KK_)                                                                                    \
-    if (gp.TC == TT && g.k == KK_) rc = (mma && TT == 3) ? launch_gradw_mma_inst<TT, KK_>(gp, prm, st) : launch_gradw_inst<TT, KK_>(gp, prm, st);
-    X(1, 1) X(1, 2) X(1, 3) X(1, 5) X(3, 1) X(3, 2) X(3, 3) X(3, 5)
-#undef X
-    }
-    if (rc) return rc;
-    if (na < 16384) {       // few entries: four lanes per entry (64 entries per CTA)
-        gradw_reduce_kernel<4><<<(int)((na + 63) / 64), 256, 0, st>>>(prm.partials, gw, shares, g.C, g.k, ld);
-    } else {
-        const int blocks = (int)((na + 255) / 256 < 4096 ? (na + 255) / 256 : 4096);
-        gradw_reduce_kernel<1><<<blocks, 256, 0, st>>>(prm.partials, gw, shares, g.C, g.k, ld);
-    }
-    return check_launch();
+    return launch_gradw_quad(gy, x, gw, g, reinterpret_cast<float*>(static_cast<char*>(ws) + INVCONV_WS_CONTROL_BYTES) + na + (size_t)g.C * g.C,
+                             st, ld);
 }
 
 template <int TA, int NGN, int NGC, int PM, int MAXT>
@@ -615,9 +586,7 @@ TensorPlan tensor_plan(int B, int C, int H, int W, int k)
 size_t tensor_wop_offset(int B, int C, int H, int W, int k)
 {
     const size_t na = sizeof(float) * (size_t)k * k * C * C;
-    const GradWPlan gp = gradw_plan(B, C, H, W, k);
-    const int shares = gp.nbc > gp.nbc_all ? gp.nbc : gp.nbc_all;
-    const size_t base = INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)C * C + (gp.ok ? na * shares : 0);
+    const size_t base = INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)C * C + na * gradw_quad_plan(B, C, H, W, k).shares;
     return (base + 255) & ~(size_t)255;
 }
 
@@ -646,14 +615,7 @@ int launch_gradw_tensor(const float* gy, const float* x, float* gw, Geom g, void
     float* partials = reinterpret_cast<float*>(static_cast<char*>(ws) + partials_offset);
     const int rc = invconv_internal::gradw_tensor_launch(gt, gy, x, partials, g, st);
     if (rc) return rc;
-    const size_t na = (size_t)g.k * g.k * g.C * g.C;
-    if (na < 16384) {
-        gradw_reduce_kernel<4><<<(int)((na + 63) / 64), 256, 0, st>>>(partials, gw, gt.S, g.C, g.k, ld);
-    } else {
-        const int blocks = (int)((na + 255) / 256 < 4096 ? (na + 255) / 256 : 4096);
-        gradw_reduce_kernel<1><<<blocks, 256, 0, st>>>(partials, gw, gt.S, g.C, g.k, ld);
-    }
-    return check_launch();
+    return launch_gradw_reduce(partials, gw, gt.S, g, st, ld);
 }
 
 // Plain or transposed solve on the tensor cores: kernel transform, operand packing, wavefront.
@@ -918,7 +880,7 @@ bool bf16_in_kernel(int B, int C, int H, int W, int k, bool bwd, bool with_gw)
     if (!pl.ok || pl.glb || ((size_t)C * H * W) % 8 != 0) return false;
     if (bwd && with_gw) {
         const GradWSmallPlan gs = gradw_small_plan(B, C, H, W, k);
-        if (gradw_separate(pl, gs, C, k)) return false;
+        if (gradw_separate(pl, gs, C, H, k, true)) return false;
     }
     return true;
 }

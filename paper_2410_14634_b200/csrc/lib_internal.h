@@ -9,6 +9,7 @@
 #include "tensor_plan.h"
 #include "line_plan.h"
 #include "warp_plan.h"
+#include "gradw_quad_plan.h"
 
 namespace invconv {
 struct LineParams;
@@ -72,14 +73,15 @@ int launch_warp_c1(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::
 int launch_gradw_small_c1(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
 int launch_masked_conv_c1(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
 int launch_warp_c2(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
-int launch_gradw_small_c2(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
 int launch_masked_conv_c2(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
 int launch_warp_c3(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
-int launch_gradw_small_c3(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
 int launch_masked_conv_c3(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
 int launch_warp_c4(int k, bool bwd, const invconv::WarpPlan& pl, const invconv::WarpParams& prm, bool ring, bool split, bool dep, cudaStream_t st);
-int launch_gradw_small_c4(int k, const invconv::GradWSmallPlan& gs, const invconv::GradWSmallParams& prm, bool dep, cudaStream_t st);
 int launch_masked_conv_c4(const float* x, const float* w, float* y, invconv::Geom g, bool dep, cudaStream_t st);
+
+// gradw_quad_lib.cu: the fp32 correlation kernel of grad_w; partial sums [pl.shares][k*k][C][C] go to `partials`.
+int gradw_quad_launch(const invconv::GradWQuadPlan& pl, const float* gy, const float* x, float* partials, invconv::Geom g,
+                      bool dependent, cudaStream_t st);
 
 // line_k*.cu: the LINE wavefront instances of one kernel side.
 int launch_line_k2(const invconv::LinePlan& pl, const invconv::LineParams& prm, bool dependent, cudaStream_t st);

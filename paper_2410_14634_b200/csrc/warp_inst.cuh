@@ -150,15 +150,6 @@ int launch_masked_conv_ck(const float* x, const float* w, float* y, Geom g, bool
         default: return INVCONV_UNSUPPORTED;                                                                               \
         }                                                                                                                  \
     }                                                                                                                      \
-    int launch_gradw_small_c##C_(int k, const GradWSmallPlan& gs, const GradWSmallParams& prm, bool dep, cudaStream_t st)  \
-    {                                                                                                                      \
-        switch (k) {                                                                                                       \
-        case 2: return launch_gradw_small_ck<C_, 2>(gs, prm, dep, st);                                                     \
-        case 3: return launch_gradw_small_ck<C_, 3>(gs, prm, dep, st);                                                     \
-        case 5: return launch_gradw_small_ck<C_, 5>(gs, prm, dep, st);                                                     \
-        default: return INVCONV_UNSUPPORTED;                                                                               \
-        }                                                                                                                  \
-    }                                                                                                                      \
     int launch_masked_conv_c##C_(const float* x, const float* w, float* y, Geom g, bool dep, cudaStream_t st)              \
     {                                                                                                                      \
         switch (g.k) {                                                                                                     \
