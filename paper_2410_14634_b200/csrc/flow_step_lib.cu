@@ -72,6 +72,8 @@ __global__ void __launch_bounds__(256) flow_mix_grad_kernel(const float* __restr
                                                             double* __restrict__ partials, int B, int C, int HW, int tiles)
 {
     extern __shared__ __align__(16) float fsm[];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float* tg = fsm;                              // [C][kMixPixels + 1]
     float* tx = tg + C * (kMixPixels + 1);        // [C][kMixPixels + 1]
     const int items = B * tiles, NE = C * C + C;
@@ -133,78 +135,190 @@ __global__ void __launch_bounds__(256) flow_mix_grad_kernel(const float* __restr
     }
 }
 
-// Sums the shares in order and forms the parameter gradients:
+// The same for up to four channels: a thread per pixel keeps all C*C + C sums in double registers (the products of two fp32 are
+// exact there), walks the pixels of its share, and the block adds its lanes' sums by shuffles.  The tile kernel above
+// left 244 of its 256 threads without an entry (C = 3: 20 us; this one 4 us).
+template <int C>
+__global__ void __launch_bounds__(256) flow_mix_grad_few_kernel(const float* __restrict__ gu, const float* __restrict__ x,
+                                                                double* __restrict__ partials, int B, int HW)
+{
+    constexpr int NE = C * C + C;
+    __shared__ double red[8][NE];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    double acc[NE];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) acc[e] = 0.0;
+    const int total = B * HW, stride = gridDim.x * blockDim.x;
+#pragma unroll 2
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        const int n = i / HW, px = i - n * HW;
+        const float* pg = gu + (size_t)n * C * HW + px;
+        const float* pxx = x + (size_t)n * C * HW + px;
+        float g[C], v[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) { g[c] = __ldg(pg + c * HW); v[c] = __ldg(pxx + c * HW); }
+#pragma unroll
+        for (int o = 0; o < C; ++o) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[o * C + c] = fma((double)g[o], (double)v[c], acc[o * C + c]);
+            acc[C * C + o] += (double)g[o];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < NE; ++e)
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int e = 0; e < NE; ++e) red[threadIdx.x >> 5][e] = acc[e];
+    }
+    __syncthreads();
+    if (threadIdx.x < NE) {
+        double a = 0.0;
+        for (int w = 0; w < 8; ++w) a += red[w][threadIdx.x];
+        partials[(size_t)blockIdx.x * NE + threadIdx.x] = a;
+    }
+}
+
+// Sums entry e of the shares: `lanes` adjacent threads (a power of two up to 32) take every lanes-th share, in order and eight loads
+// in flight, and are combined in a fixed order.  Every lane of the group returns the total.
+__device__ __forceinline__ double sum_shares(const double* __restrict__ partials, int shares, int NE, int e, int lane, int lanes)
+{
+    double a = 0.0;
+    for (int s0 = lane; s0 < shares; s0 += 8 * lanes) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = s0 + q * lanes < shares ? __ldcg(partials + (size_t)(s0 + q * lanes) * NE + e) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a += v[q];
+    }
+    for (int o = 1; o < lanes; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+// Many entries: the sums over the shares on many CTAs (eight lanes per entry), in place of the first share.
+__global__ void __launch_bounds__(256) flow_mix_grad_sum_kernel(const double* __restrict__ partials, double* __restrict__ G, int shares, int NE)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int e = (blockIdx.x * 256 + threadIdx.x) >> 3;
+    const double a = sum_shares(partials, shares, NE, e < NE ? e : NE - 1, threadIdx.x & 7, 8);
+    if (e < NE && (threadIdx.x & 7) == 0) G[e] = a;
+}
+
+// Sums the shares in order (unless `summed`: partials then holds the sums) and forms the parameter gradients:
 //   grad_V[o][c] = s[c] * G1[o][c] + b[c] * g0[o];  grad_s[c] = sum_o V[o][c] * G1[o][c];  grad_b[c] = sum_o V[o][c] * g0[o].
-__global__ void __launch_bounds__(256) flow_mix_grad_final_kernel(const double* __restrict__ partials, int shares,
-                                                                  const float* __restrict__ V, const float* __restrict__ s,
-                                                                  const float* __restrict__ b, float* __restrict__ grad_V,
-                                                                  float* __restrict__ grad_s, float* __restrict__ grad_b, int C)
+__global__ void __launch_bounds__(1024) flow_mix_grad_final_kernel(const double* __restrict__ partials, int shares, int summed,
+                                                                   const float* __restrict__ V, const float* __restrict__ s,
+                                                                   const float* __restrict__ b, float* __restrict__ grad_V,
+                                                                   float* __restrict__ grad_s, float* __restrict__ grad_b, int C, int lanes)
 {
     extern __shared__ __align__(16) double fsmd[];
     double* G = fsmd;                 // [C*C + C]
     const int NE = C * C + C;
-    for (int e = threadIdx.x; e < NE; e += blockDim.x) {
-        double a = 0.0;
-        for (int sh = 0; sh < shares; ++sh) a += __ldcg(partials + (size_t)sh * NE + e);
-        G[e] = a;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (summed || shares == 0) {
+        for (int e = threadIdx.x; e < NE; e += blockDim.x) G[e] = shares == 0 ? 0.0 : __ldcg(partials + e);
+    } else {
+        const int per = blockDim.x / lanes, l = threadIdx.x & (lanes - 1), g = threadIdx.x / lanes;
+        for (int e0 = 0; e0 < NE; e0 += per) {
+            const int e = e0 + g;
+            const double a = sum_shares(partials, shares, NE, e < NE ? e : NE - 1, l, lanes);
+            if (e < NE && l == 0) G[e] = a;
+        }
     }
     __syncthreads();
     for (int e = threadIdx.x; e < C * C; e += blockDim.x) {
         const int o = e / C, c = e - o * C;
         grad_V[e] = (float)((double)__ldg(s + c) * G[e] + (double)__ldg(b + c) * G[C * C + o]);
     }
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
+    // a warp per channel: the sum over o in a fixed order
+    for (int c = threadIdx.x >> 5; c < C; c += blockDim.x >> 5) {
         double gs = 0.0, gb = 0.0;
-        for (int o = 0; o < C; ++o) {
+        for (int o = threadIdx.x & 31; o < C; o += 32) {
             const double v = (double)__ldg(V + o * C + c);
             gs += v * G[o * C + c];
             gb += v * G[C * C + o];
         }
-        grad_s[c] = (float)gs;
-        grad_b[c] = (float)gb;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) { gs += __shfl_xor_sync(0xffffffffu, gs, o); gb += __shfl_xor_sync(0xffffffffu, gb, o); }
+        if ((threadIdx.x & 31) == 0) { grad_s[c] = (float)gs; grad_b[c] = (float)gb; }
     }
 }
 
 // logdet[0] = H*W * ( -sum_c log|w[c][c][k-1][k-1]| + sum_c log|s[c]| + log|det V| ), in double; the determinant by
-// Gaussian elimination with partial pivoting in shared memory (one CTA, C <= 128).
-__global__ void __launch_bounds__(128) flow_logdet_kernel(const float* __restrict__ w, const float* __restrict__ s,
+// Gaussian elimination with partial pivoting in shared memory (one CTA, C <= 128): warp 0 finds the pivot among the rows
+// not used yet (rows stay where they are, `used` marks them), then all threads eliminate.  Reads only the parameters, so it is
+// launched dependently behind the solve and runs beside it; it waits for the solve before it ends, which keeps the stream's order.
+__global__ void __launch_bounds__(256) flow_logdet_kernel(const float* __restrict__ w, const float* __restrict__ s,
                                                           const float* __restrict__ V, float* __restrict__ logdet,
                                                           int C, int H, int W, int K)
 {
     extern __shared__ __align__(16) double dsm[];
     double* M = dsm;                  // [C][C]
+    double* pivot = M + C * C;        // [C]
+    __shared__ unsigned char used[128];
     __shared__ int piv;
-    __shared__ double acc;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int e = tid; e < C * C; e += blockDim.x) M[e] = (double)__ldg(V + e);
-    if (tid == 0) {
-        double a = 0.0;
-        for (int c = 0; c < C; ++c)
-            a += log(fabs((double)__ldg(s + c))) - log(fabs((double)__ldg(w + ((size_t)(c * C + c) * K + (K - 1)) * K + (K - 1))));
-        acc = a;
-    }
+    if (tid < 128) used[tid] = 0;
     __syncthreads();
     for (int j = 0; j < C; ++j) {
-        if (tid == 0) {
-            int best = j;
-            double bv = fabs(M[j * C + j]);
-            for (int i = j + 1; i < C; ++i)
-                if (fabs(M[i * C + j]) > bv) { bv = fabs(M[i * C + j]); best = i; }
-            piv = best;
+        if (tid < 32) {
+            double bv = -1.0;
+            int best = 0;
+            for (int i = lane; i < C; i += 32)
+                if (!used[i] && fabs(M[i * C + j]) > bv) { bv = fabs(M[i * C + j]); best = i; }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, best, o);
+                if (ov > bv || (ov == bv && oi < best)) { bv = ov; best = oi; }
+            }
+            if (lane == 0) { piv = best; used[best] = 1; pivot[j] = bv; }
         }
         __syncthreads();
-        if (piv != j)
-            for (int c = tid; c < C; c += blockDim.x) { const double t = M[j * C + c]; M[j * C + c] = M[piv * C + c]; M[piv * C + c] = t; }
-        __syncthreads();
-        const double d = M[j * C + j];
-        if (tid == 0) acc += log(fabs(d));
-        for (int i = j + 1 + tid; i < C; i += blockDim.x) {
-            const double f = M[i * C + j] / d;
-            for (int c = j + 1; c < C; ++c) M[i * C + c] -= f * M[j * C + c];
+        const int pr = piv;
+        const double inv = 1.0 / M[pr * C + j];
+        const int cols = C - j - 1;
+        for (int i = tid >> 5; i < C; i += blockDim.x >> 5) {
+            if (used[i]) continue;
+            const double f = M[i * C + j] * inv;
+            for (int c = lane; c < cols; c += 32) M[i * C + j + 1 + c] -= f * M[pr * C + j + 1 + c];
         }
         __syncthreads();
     }
-    if (tid == 0) logdet[0] = (float)((double)(H * W) * acc);
+    if (tid < 32) {
+        double a = 0.0;
+        for (int c = lane; c < C; c += 32)
+            a += log(fabs((double)__ldg(s + c))) - log(fabs((double)__ldg(w + ((size_t)(c * C + c) * K + (K - 1)) * K + (K - 1)))) + log(pivot[c]);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) logdet[0] = (float)((double)(H * W) * a);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launch with programmatic dependence on the kernel before: every kernel launched this way waits for it (griddepcontrol.wait).
+template <typename... P, typename... A>
+int launch_dependent(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args)
+{
+    const int rc = invconv_internal::set_smem_limit(kern, smem);
+    if (rc) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
+    return check_launch();
 }
 
 struct Scratch {
@@ -280,10 +394,10 @@ FlowScratch flow_scratch(int B, int C, int H, int W, int k)
     f.layer = up256(invconv_workspace_bytes(B > 0 ? B : 1, C, H, W, k) + INVCONV_WS_CONTROL_BYTES);
     f.act = up256(sizeof(float) * (size_t)B * C * H * W);
     f.tiles = (H * W + kMixPixels - 1) / kMixPixels;
-    f.shares = invconv_internal::sm_count() * 2;
+    f.shares = invconv_internal::sm_count();
     if (f.shares > B * f.tiles) f.shares = B * f.tiles;
     if (f.shares < 1) f.shares = 1;
-    f.part = up256(sizeof(double) * ((size_t)C * C + C) * f.shares);
+    f.part = up256(sizeof(double) * ((size_t)C * C + C) * (f.shares + 1));
     f.total = f.layer + f.act + f.part;
     return f;
 }
@@ -327,12 +441,7 @@ int invconv_flow_step_forward_ws(const float* y, const float* w, const float* s,
         if (rc) return rc;
     }
     if (logdet) {
-        auto kern = flow_logdet_kernel;
-        const size_t sm = sizeof(double) * (size_t)C * C;
-        rc = invconv_internal::set_smem_limit(kern, sm);
-        if (rc) return rc;
-        kern<<<1, 128, sm, st>>>(w, s, V, logdet, C, H, W, k);
-        return check_launch();
+        return launch_dependent(flow_logdet_kernel, 1, 256, sizeof(double) * ((size_t)C * C + C), st, w, s, V, logdet, C, H, W, k);
     }
     return INVCONV_OK;
 }
@@ -371,24 +480,36 @@ int invconv_flow_step_backward_ws(const float* grad_u, const float* x, const flo
             rc = invconv_backward_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, workspace, f.layer, stream);
         }
         if (rc) return rc;
-        const size_t sm = sizeof(float) * 2 * (size_t)C * (kMixPixels + 1);
-        auto kern = flow_mix_grad_kernel;
-        rc = invconv_internal::set_smem_limit(kern, sm);
-        if (rc) return rc;
-        kern<<<shares, 256, sm, st>>>(grad_u, x, partials, B, C, HW, f.tiles);
-        rc = check_launch();
+        if (C <= 4) {
+            switch (C) {
+            case 1: rc = launch_dependent(flow_mix_grad_few_kernel<1>, shares, 256, 0, st, grad_u, x, partials, B, HW); break;
+            case 2: rc = launch_dependent(flow_mix_grad_few_kernel<2>, shares, 256, 0, st, grad_u, x, partials, B, HW); break;
+            case 3: rc = launch_dependent(flow_mix_grad_few_kernel<3>, shares, 256, 0, st, grad_u, x, partials, B, HW); break;
+            default: rc = launch_dependent(flow_mix_grad_few_kernel<4>, shares, 256, 0, st, grad_u, x, partials, B, HW); break;
+            }
+        } else {
+            rc = launch_dependent(flow_mix_grad_kernel, shares, 256, sizeof(float) * 2 * (size_t)C * (kMixPixels + 1), st, grad_u, x, partials,
+                                  B, C, HW, f.tiles);
+        }
         if (rc) return rc;
     } else {
         rc = invconv_backward_ws(grad_u, x, w, grad_y, grad_w, 0, C, H, W, k, nullptr, 0, stream);   // zeroes grad_w
         if (rc) return rc;
         shares = 0;
     }
-    const size_t smf = sizeof(double) * ((size_t)C * C + C);
-    auto kf = flow_mix_grad_final_kernel;
-    rc = invconv_internal::set_smem_limit(kf, smf);
-    if (rc) return rc;
-    kf<<<1, 256, smf, st>>>(partials, shares, V, s, b, grad_V, grad_s, grad_b, C);
-    return check_launch();
+    // few entries: summed by the final kernel itself, as many lanes per entry as its 1024 threads give; many: on CTAs of their own
+    const int NE = C * C + C;
+    const bool separate = NE > 512 && shares > 0;
+    if (separate) {
+        double* sums = partials + (size_t)NE * shares;
+        rc = launch_dependent(flow_mix_grad_sum_kernel, (NE * 8 + 255) / 256, 256, 0, st, partials, sums, shares, NE);
+        if (rc) return rc;
+        partials = sums;
+    }
+    int lanes = 1;
+    while (lanes < 32 && NE * lanes * 2 <= 1024) lanes *= 2;
+    return launch_dependent(flow_mix_grad_final_kernel, 1, 1024, sizeof(double) * (size_t)NE, st, partials, shares, separate ? 1 : 0, V, s, b,
+                            grad_V, grad_s, grad_b, C, lanes);
 }
 
 int invconv_flow_step_backward(const float* grad_u, const float* x, const float* w, const float* s, const float* b,

@@ -680,6 +680,15 @@ size_t workspace_bytes_for(int path, int B, int C, int H, int W, int k)
     return 0;
 }
 
+// grad_w of the team and tensor families from the solved grad_y.
+int launch_gradw_many(int path, const float* gy, const float* x, float* gw, Geom g, void* ws, cudaStream_t st, const LogdetFuse& ld)
+{
+    const size_t na = sizeof(float) * (size_t)g.k * g.k * g.C * g.C;
+    const size_t off = path == INVCONV_PATH_TENSOR ? tensor_gradw_offset(g.B, g.C, g.H, g.W, g.k)
+                                                   : INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)g.C * g.C;
+    return launch_gradw_tensor(gy, x, gw, g, ws, off, st, ld);
+}
+
 // `logdet_out` (optional): the layer's log-det, written by the forward kernels themselves where they have a
 // warp to spare (warp family; the kernel transform of the team and tensor families), else by its own launch.
 int launch_forward(int path, const float* y, const float* w, float* x, Geom g,
@@ -747,11 +756,7 @@ int launch_backward(int path, const float* gx, const float* x, const float* w, f
             const int rc = launch_team(true, gx, w, gy, g, ws, st);
             if (rc) return rc;
         }
-        if (gw) {
-            const size_t na = sizeof(float) * (size_t)g.k * g.k * g.C * g.C;
-            return launch_gradw_tensor(gy, x, gw, g, ws, INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)g.C * g.C, st, ld);
-        }
-        return INVCONV_OK;
+        return gw ? launch_gradw_many(path, gy, x, gw, g, ws, st, ld) : INVCONV_OK;
     }
     case INVCONV_PATH_TENSOR: {
         if (g.B > 0) {
@@ -771,8 +776,7 @@ int launch_backward(int path, const float* gx, const float* x, const float* w, f
             }
             if (rc) return rc;
         }
-        if (gw) return launch_gradw_tensor(gy, x, gw, g, ws, tensor_gradw_offset(g.B, g.C, g.H, g.W, g.k), st, ld);
-        return INVCONV_OK;
+        return gw ? launch_gradw_many(path, gy, x, gw, g, ws, st, ld) : INVCONV_OK;
     }
     default:
         return INVCONV_UNSUPPORTED;
@@ -911,9 +915,15 @@ int warp_step_forward(const float* y, const float* w, const float* s, const floa
 int warp_step_backward(const float* grad_u, const float* x, const float* w, const float* s, const float* V,
                        float* grad_y, float* grad_w, Geom g, void* ws, cudaStream_t st)
 {
-    if (resolve_path(g.B, g.C, g.H, g.W, g.k) != INVCONV_PATH_WARP) return INVCONV_UNSUPPORTED;
+    const int path = resolve_path(g.B, g.C, g.H, g.W, g.k);
     WarpMix mix;
     mix.V = V; mix.s = s; mix.grad_in = true;
+    if (path != INVCONV_PATH_WARP) {
+        // the line wavefront takes the neighbours with the kernel: its right-hand side enters through A_0 diag(s) V^T
+        if (path == INVCONV_PATH_GENERIC || !line_preferred(g.B, g.C, g.H, g.W, g.k)) return INVCONV_UNSUPPORTED;
+        const int rc = launch_line(true, grad_u, w, grad_y, g, st, &mix);
+        return rc ? rc : launch_gradw_many(path, grad_y, x, grad_w, g, ws, st, LogdetFuse{});
+    }
     return launch_warp(true, grad_u, w, grad_y, x, grad_w, g, ws, st, &mix);
 }
 
