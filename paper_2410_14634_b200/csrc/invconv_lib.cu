@@ -249,7 +249,8 @@ int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cu
     prm.vec = (g.W % 4 == 0 && (ptrs & (bf16 ? 7 : 15)) == 0) ? 1 : 0;
     prm.ncw = pl.ncw; prm.niow = pl.niow;
     prm.bk_warps = pl.bk_warps; prm.bk_parts = pl.bk_parts; prm.bk_per = pl.bk_per; prm.div_bk = make_fast_div((unsigned)pl.bk_warps);
-    prm.off_dummy = pl.off_dummy; prm.off_ring = pl.off_ring; prm.off_a = pl.off_a; prm.off_w = pl.off_w; prm.off_li = pl.off_li;
+    prm.pieces = pl.pieces;
+    prm.off_dummy = pl.off_dummy; prm.off_y = pl.off_y; prm.off_ring = pl.off_ring; prm.off_a = pl.off_a; prm.off_w = pl.off_w; prm.off_li = pl.off_li;
     if (mix) {
         prm.mix_V = mix->V; prm.mix_s = mix->s; prm.mix_b = mix->b;
         prm.mix_out = bwd ? nullptr : mix->u_out;

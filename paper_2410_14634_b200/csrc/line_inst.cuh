@@ -16,7 +16,7 @@ int launch_line_inst(const invconv::LinePlan& pl, const invconv::LineParams& prm
     if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(pl.grid);
-    cfg.blockDim = dim3((pl.ncw + pl.niow) * 32);
+    cfg.blockDim = dim3((pl.ncw + 2 * pl.niow) * 32);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -11,9 +11,9 @@
 // vectors to the pending sums.  Each value is read once and used for K taps; nothing but the newest pixel of each
 // row is ever exchanged, so shared memory holds no image and the image size is not limited by it.
 //
-// Reading and writing global memory is the job of separate I/O warps: a ring of 32 columns per row takes the right-hand
-// side in chunks of eight columns, requested three and placed two chunks ahead of the wavefront; the solution overwrites it in
-// place and leaves one chunk behind.  Images taller than a CTA's rows are walked in bands from top to bottom; the K-1 rows above
+// Reading and writing global memory is the job of separate I/O warps: a ring of 64 columns per row and channel takes the
+// right-hand side in chunks of eight columns (16-byte asynchronous copies) two chunks ahead of the wavefront; the solution
+// overwrites it in place and leaves one chunk behind.  Images taller than a CTA's rows are walked in bands from top to bottom; the K-1 rows above
 // a band are "halo" rows whose threads publish the values that the band before wrote to global memory.  Images and bands
 // follow one another on one virtual column axis with zero columns between them, so a CTA with several images pays the ramp
 // of the wavefront once.
@@ -42,7 +42,7 @@ namespace invconv {
 namespace line_detail {
 
 using u64 = unsigned long long;
-constexpr int kRing = 32;
+constexpr int kRing = 64, kChan = kRing + 4;      // columns of a row and channel in the ring, and floats between channels
 
 // The NB input channels of a slice as NV operands: packed pairs for even NB.
 template <int NB, bool PACK = (NB % 2 == 0)>
@@ -53,6 +53,7 @@ struct Vec {
     static __device__ __forceinline__ float sum(T a) { return a; }
     static __device__ __forceinline__ T zero() { return 0.f; }
     static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+    static __device__ __forceinline__ T pick(const float (&f)[NB], int q) { return f[q]; }
     template <bool AL16>
     static __device__ __forceinline__ void load(const float* p, T (&v)[NV])
     {
@@ -100,6 +101,7 @@ struct Vec<NB, true> {
         asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
         return d;
     }
+    static __device__ __forceinline__ T pick(const float (&f)[NB], int q) { return pair(f[2 * q], f[2 * q + 1]); }
     template <bool AL16>
     static __device__ __forceinline__ void load(const float* p, T (&v)[NV])
     {
@@ -200,21 +202,24 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     constexpr int NV = V::NV, KK = K * K, KM = K - 1;
     constexpr int NPEND = 2 * K - 3;                   // pending sums: the next columns that solved pixels reach
     constexpr int CSB = S * NB, CS = (CSB + 3) / 4 * 4;          // channels of a pixel in shared memory, padded to 16 bytes
-    constexpr int RS = line_row_stride(kRing, CS);
     constexpr bool AL16 = S == 1 || NB % 4 == 0;
-    constexpr int UNR = PR * NV * KK <= 64 ? 4 : 2;    // steps per turn of the loop
+    constexpr int UNR = 2;    // steps per turn of the loop
     extern __shared__ __align__(128) float sm[];
-    __shared__ unsigned long long bars[4];             // chunk ready [2], chunk done [2]
+    __shared__ unsigned long long bars[6];             // chunk ready [2], chunk done [2], chunk read for storing [2]
     __shared__ int gave_up_flag;
     volatile int* gave_up = &gave_up_flag;
     const int C = p.C, H = p.H, W = p.W, HW = H * W;
     const int HBt = p.HB + p.halo;
     const int exrow = (HBt + KM + PR) * CS;
     float* EX = sm;                                    // [2][HBt + K-1 + PR][CS]: newest pixel of every row, by step
-    float* RG = sm + p.off_ring;                       // [HBt][32 columns][CS] (row stride RS)
+    float* EY = sm + p.off_y;                          // [2][HBt + PR][CS]: right-hand side of the next pixel of every row, by step parity
+    float* RG = sm + p.off_ring;                       // [HBt][C][64 columns]
+    const int rm = p.rot ? kRing - 1 : 0;              // slot of virtual column vc: (vc ^ rm) & 63, which is memory order either way
+    const int yrow = (HBt + PR) * CS, RS = C * kChan;
     float* As = sm + p.off_a;
     unsigned long long* ready_bar = bars;
     unsigned long long* done_bar = bars + 2;
+    unsigned long long* read_bar = bars + 4;
     float* const dummy = sm + p.off_dummy;             // scratch words for lanes without a pixel
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int NT = blockDim.x, nct = p.ncw * 32;
@@ -227,12 +232,12 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     if (tid == 0) {
         mbar_init(ready_bar, p.niow * 32); mbar_init(ready_bar + 1, p.niow * 32);
         mbar_init(done_bar, p.ncw); mbar_init(done_bar + 1, p.ncw);
+        mbar_init(read_bar, p.niow); mbar_init(read_bar + 1, p.niow);
         gave_up_flag = 0;
         fence_mbar_init();
     }
     for (int i = tid; i < 2 * exrow; i += NT) EX[i] = 0.f;
-    if (C < CSB)                                       // channels beyond C meet zero weights but must not be NaN
-        for (int i = tid; i < HBt * RS; i += NT) RG[i] = 0.f;
+    for (int i = tid; i < 2 * yrow; i += NT) EY[i] = 0.f;          // channels beyond C meet zero weights but must not be NaN
     for (int i = p.off_a + tid; i < p.off_w; i += NT) sm[i] = 0.f;     // As and li
     __syncthreads();
     // everything above touched no global memory; from here on the predecessor kernel's results are needed
@@ -240,18 +245,17 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---------------------------------------------------------------- I/O
-    // A piece is four columns of one (row, channel), half a chunk; a thread owns the same BV pieces of every chunk, so it may
-    // place a chunk where it has just stored one.  Row r is floor(r/8) chunks behind row 0 when read, ceil(r/8) when
-    // stored.  Loads are unconditional (from a valid address) and kept as raw bits until they are placed, so that all of
-    // a thread's requests are in flight at once.
-    constexpr int BV = line_pieces(NB, S);
-    const bool io_warp = warp >= p.ncw;
-    const int io = tid - nct, nio = p.niow * 32;
+    // Half of the I/O warps load, half store (together their loop outgrew the instruction cache: 2500 cycles a chunk against 1000
+    // and 1300 apart).  A piece is four columns of one (row, channel), half a chunk; a thread owns the same BV pieces of
+    // every chunk.  Row r is floor(r/8) chunks behind row 0 when read, ceil(r/8) when stored.
+    constexpr int BV = kLinePieces;                    // at most; p.pieces of them are used
+    const bool io_warp = warp >= p.ncw, loader = warp < p.ncw + p.niow;
+    const int nio = p.niow * 32, io = tid - nct - (loader ? 0 : nio);
     const int half4 = 4 * (io & 1), sgn = p.rot ? -1 : 1;
     int ring_off[BV], gofs[BV], row[BV];
-    // per piece: column within its segment, segment, and the element of the segment row's first column (-1: no such row) --
-    // of the chunk requested next and of the chunk stored next
-    int rcol[BV], rseg[BV], rbase[BV], scol[BV], sseg[BV], sbase[BV];
+    // per piece, of the chunk moved next: column within its segment, segment, and the element of the segment row's first column
+    // (-1: no such row)
+    int pcol[BV], pseg[BV], pbase[BV];
     auto seg_base = [&](int b, int seg) -> int {
         if (seg >= nseg) return -1;
         const int i = p.nbands == 1 ? seg : fast_div(seg, p.div_nb), band = seg - i * p.nbands;
@@ -265,12 +269,11 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
             const int rc = (io + b * nio) >> 1, rr = fast_div(rc, p.div_c), c = rc - rr * C, r = rr - p.halo;
             const bool ok = rr < HBt;
             row[b] = ok ? r : -1000000;                // never inside the image
-            ring_off[b] = ok ? rr * RS + c : 0;
+            ring_off[b] = ok ? rr * RS + c * kChan : 0;
             gofs[b] = ok ? c * HW + (p.rot ? HW - 1 - r * W : r * W) : 0;
-            rcol[b] = half4 - (ok ? 8 * (r >> 3) : 0); scol[b] = half4 - (ok ? 8 * ((r + 7) >> 3) : 0);
-            rseg[b] = 0; sseg[b] = 0;
-            rbase[b] = seg_base(b, 0);
-            sbase[b] = r < 0 ? -1 : rbase[b];
+            pcol[b] = half4 - (ok ? 8 * ((loader ? r : r + 7) >> 3) : 0);
+            pseg[b] = 0;
+            pbase[b] = r < 0 && !loader ? -1 : seg_base(b, 0);
         }
     }
     auto advance = [&](int b, int& col, int& seg, int& base) {
@@ -283,14 +286,20 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     auto copy = [&](int t) {
 #pragma unroll
         for (int b = 0; b < BV; ++b) {
-            const bool have = rbase[b] >= 0 && rcol[b] >= 0;
-            const int vc = 8 * (t - (row[b] >> 3)) + half4;
-            const float* g = reinterpret_cast<const float*>(row[b] < 0 ? p.out : p.rhs) + (have ? rbase[b] + sgn * rcol[b] : safe);
-            float* d = row[b] > -1000 ? RG + ring_off[b] + (vc & (kRing - 1)) * CS : dummy;
-            const int ds = row[b] > -1000 ? CS : 0, left = have ? W - rcol[b] : 0;
+            if (b >= p.pieces) break;                  // uniform
+            const bool have = pbase[b] >= 0 && pcol[b] >= 0;
+            const int vc = 8 * (t - (row[b] >> 3)) + half4, left = have ? W - pcol[b] : 0;
+            const float* g = reinterpret_cast<const float*>(row[b] < 0 ? p.out : p.rhs) + (left > 0 ? pbase[b] + sgn * pcol[b] : safe);
+            float* d = RG + ring_off[b];
+            if (row[b] > -1000) {
+                if (p.vec) {
+                    cp_async_f32x4(d + (((vc ^ rm) & (kRing - 1)) & ~3), left > 0 && p.rot ? g - 3 : g, left > 0);
+                } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) cp_async_f32(d + j * ds, j < left ? g + sgn * j : g, j < left);
-            advance(b, rcol[b], rseg[b], rbase[b]);
+                    for (int j = 0; j < 4; ++j) cp_async_f32(d + (((vc + j) ^ rm) & (kRing - 1)), j < left ? g + sgn * j : g, j < left);
+                }
+            }
+            advance(b, pcol[b], pseg[b], pbase[b]);
         }
     };
     // bf16: requested into registers a chunk ahead, widened when placed
@@ -298,8 +307,9 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     auto request = [&](unsigned (&v)[4 * BV]) {
 #pragma unroll
         for (int b = 0; b < BV; ++b) {
-            const int nv = rbase[b] >= 0 && rcol[b] >= 0 ? min(max(W - rcol[b], 0), 4) : 0;
-            const int f = rbase[b] + sgn * rcol[b];
+            if (b >= p.pieces) break;
+            const int nv = pbase[b] >= 0 && pcol[b] >= 0 ? min(max(W - pcol[b], 0), 4) : 0;
+            const int f = pbase[b] + sgn * pcol[b];
             rnv[b] = nv;
             const __nv_bfloat16* src = reinterpret_cast<const __nv_bfloat16*>(row[b] < 0 ? p.out : p.rhs);
             if (p.vec) {
@@ -309,73 +319,84 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
 #pragma unroll
                 for (int j = 0; j < 4; ++j) v[4 * b + j] = reinterpret_cast<const unsigned short*>(src)[j < nv ? f + sgn * j : safe];
             }
-            advance(b, rcol[b], rseg[b], rbase[b]);
+            advance(b, pcol[b], pseg[b], pbase[b]);
         }
     };
     auto place = [&](const unsigned (&v)[4 * BV], int t) {
 #pragma unroll
         for (int b = 0; b < BV; ++b) {
+            if (b >= p.pieces) break;
             const int vc = 8 * (t - (row[b] >> 3)) + half4;
             unsigned u[4];
-            if (p.vec) { u[3] = v[4 * b + 1] & 0xffff0000u; u[2] = v[4 * b + 1] << 16; u[1] = v[4 * b] & 0xffff0000u; u[0] = v[4 * b] << 16; }
-            else {
+            if (row[b] <= -1000) continue;
+            float* d = RG + ring_off[b];
+            if (p.vec) {                                 // memory order is slot order
+                u[3] = v[4 * b + 1] & 0xffff0000u; u[2] = v[4 * b + 1] << 16; u[1] = v[4 * b] & 0xffff0000u; u[0] = v[4 * b] << 16;
+                if (rnv[b] == 0) u[0] = u[1] = u[2] = u[3] = 0u;
+                *reinterpret_cast<uint4*>(d + (((vc ^ rm) & (kRing - 1)) & ~3)) = make_uint4(u[0], u[1], u[2], u[3]);
+            } else {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) u[j] = v[4 * b + j] << 16;
+                for (int j = 0; j < 4; ++j)
+                    d[((vc + j) ^ rm) & (kRing - 1)] = j < rnv[b] ? __uint_as_float(v[4 * b + j] << 16) : 0.f;
             }
-            float* d = row[b] > -1000 ? RG + ring_off[b] + (vc & (kRing - 1)) * CS : dummy;
-            const int ds = row[b] > -1000 ? CS : 0;
-            const bool flip = p.vec && p.rot;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) d[j * ds] = j < rnv[b] ? __uint_as_float(flip ? u[3 - j] : u[j]) : 0.f;
         }
     };
     // u = V (s x + b) of the flow step for one channel of one pixel
     auto mixed = [&](const float* px, int c) -> float {
         float u = 0.f;
-        for (int m = 0; m < C; ++m) u = fmaf(__ldg(p.mix_V + c * C + m), fmaf(__ldg(p.mix_s + m), px[m], __ldg(p.mix_b + m)), u);
+        for (int m = 0; m < C; ++m) u = fmaf(__ldg(p.mix_V + c * C + m), fmaf(__ldg(p.mix_s + m), px[m * kChan], __ldg(p.mix_b + m)), u);
         return u;
     };
-    auto store = [&](int t) {
-        float f[BV][4];
+    auto hand_back = [&](int t) {                      // the finished chunk has been read
+        __syncwarp();
+        if (lane == 0) mbar_arrive(read_bar + (t & 1));
+    };
+    auto store = [&](int t) {                          // at time t: what interval t-1 finished
 #pragma unroll
-        for (int b = 0; b < BV; ++b) {
-            const int vc = 8 * (t - ((row[b] + 7) >> 3)) + half4;
-            const float* px = RG + ring_off[b] + (vc & (kRing - 1)) * CS;
+        for (int b0 = 0; b0 < BV; b0 += 4) {
+        if (b0 >= p.pieces) break;
+        float4 f[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) f[b][j] = px[j * CS];
+        for (int q = 0; q < 4; ++q) {
+            const int vc = 8 * (t - 1 - ((row[b0 + q] + 7) >> 3)) + half4;
+            f[q] = *reinterpret_cast<const float4*>(RG + ring_off[b0 + q] + (((vc ^ rm) & (kRing - 1)) & ~3));      // memory order
         }
+        if (p.mix_out == nullptr && b0 + 4 >= p.pieces) hand_back(t);
 #pragma unroll
-        for (int b = 0; b < BV; ++b) {
-            const int nv = sbase[b] >= 0 && scol[b] >= 0 ? min(max(W - scol[b], 0), 4) : 0;
-            int i = sbase[b] + sgn * scol[b];
-            advance(b, scol[b], sseg[b], sbase[b]);
-            if (row[b] < 0) sbase[b] = -1;             // halo rows are not stored
+        for (int q = 0; q < 4; ++q) {
+            const int b = b0 + q;
+            const int nv = pbase[b] >= 0 && pcol[b] >= 0 ? min(max(W - pcol[b], 0), 4) : 0;
+            const int i = pbase[b] + sgn * pcol[b];
+            advance(b, pcol[b], pseg[b], pbase[b]);
+            if (row[b] < 0) pbase[b] = -1;             // halo rows are not stored
             if (nv == 0) continue;
             if (p.vec) {
-                float g[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) g[j] = p.rot ? f[b][3 - j] : f[b][j];
-                if (p.rot) i -= 3;
+                const int lo = p.rot ? i - 3 : i;
                 if (p.bf16) {
-                    const __nv_bfloat162 lo = __floats2bfloat162_rn(g[0], g[1]), hi = __floats2bfloat162_rn(g[2], g[3]);
-                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + i) =
-                        make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+                    const __nv_bfloat162 a = __floats2bfloat162_rn(f[q].x, f[q].y), c = __floats2bfloat162_rn(f[q].z, f[q].w);
+                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + lo) =
+                        make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&c));
                 } else {
-                    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + i) = make_float4(g[0], g[1], g[2], g[3]);
+                    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + lo) = f[q];
                 }
             } else {
+                const float e[4] = {f[q].x, f[q].y, f[q].z, f[q].w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < 4; ++j) {
+                    const float v = p.rot ? e[3 - j] : e[j];
                     if (j < nv) {
-                        if (p.bf16) reinterpret_cast<__nv_bfloat16*>(p.out)[i + sgn * j] = __float2bfloat16_rn(f[b][j]);
-                        else reinterpret_cast<float*>(p.out)[i + sgn * j] = f[b][j];
+                        if (p.bf16) reinterpret_cast<__nv_bfloat16*>(p.out)[i + sgn * j] = __float2bfloat16_rn(v);
+                        else reinterpret_cast<float*>(p.out)[i + sgn * j] = v;
                     }
+                }
             }
-            if (p.mix_out != nullptr) {                  // forward only
-                const int c = ring_off[b] % RS, vc = 8 * (t - ((row[b] + 7) >> 3)) + half4;
-                for (int j = 0; j < nv; ++j) p.mix_out[i + j] = mixed(RG + ring_off[b] - c + ((vc + j) & (kRing - 1)) * CS, c);
+            if (p.mix_out != nullptr) {                  // forward only: slots are virtual columns
+                const int rr = row[b] + p.halo, c = (ring_off[q] - rr * RS) / kChan, vc = 8 * (t - 1 - ((row[b] + 7) >> 3)) + half4;
+                for (int j = 0; j < nv; ++j) p.mix_out[i + j] = mixed(RG + rr * RS + ((vc + j) & (kRing - 1)), c);
             }
         }
+        }
+        if (p.mix_out != nullptr) hand_back(t);
     };
     if (!io_warp) {
         {
@@ -427,7 +448,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         for (int i = 0; i < PR; ++i) { band[i] = 0; width[i] = row_width(i, 0); }
         // rows of this warp: the warp works in an interval while any of them is between K-1 columns before its first and its last
         const int g_lo = fast_div((warp * 32) / S, p.div_c), g_hi = fast_div((warp * 32 + 31) / S, p.div_c);
-        const int t_lo = max(0, (g_lo * PR - p.halo - KM) >> 3), t_hi = (VC + min(g_hi * PR + PR - 1, HBt - 1) - p.halo + 7) >> 3;
+        const int t_lo = max(0, (g_lo * PR - p.halo - (KM > 2 ? KM : 2)) >> 3), t_hi = (VC + min(g_hi * PR + PR - 1, HBt - 1) - p.halo + 7) >> 3;
         // column within the segment of each row's pixel in the warp's first step; negative before its first column
         int col[PR];
 #pragma unroll
@@ -437,7 +458,9 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         for (int i = 0; i < PR; ++i) pub[i] = live && sl == 0 && rr0 + i < HBt;
         float* const ex_rd = EX + (rr0 + KM) * CS + sl * NB;
         float* const ex_wr = EX + (rr0 + KM) * CS + a;
-        float* const ring0 = RG + rr0 * RS;
+        float* const ring0 = RG + rr0 * RS + a * kChan;
+        float* const ey_rd = EY + rr0 * CS + sl * NB;
+        float* const ey_wr = EY + rr0 * CS + a;
         // One step; `odd`: its parity, HALO: the CTA walks bands.  No branches: on the dependent path of a step each cost 15 to
         // 20 cycles (a C = 3, k = 3 step went from 310 to 150 cycles).
         auto step = [&](int s, bool odd, auto halo_tag) {
@@ -450,7 +473,10 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
             for (int m = 0; m < PR + KM; ++m) V::template load<AL16>(ex_rd + rd + (PR - 1 - m) * CS, v[m]);
 #pragma unroll
             for (int i = 0; i < PR; ++i)
-                V::template load<AL16>(ring0 + i * RS + ((s - (rr0 + i - p.halo) + 1) & (kRing - 1)) * CS + sl * NB, rh[i]);
+                V::template load<AL16>(ey_rd + (odd ? 0 : yrow) + i * CS, rh[i]);
+            float y2[PR];                              // own channel's right-hand side two columns ahead, published for the next step
+#pragma unroll
+            for (int i = 0; i < PR; ++i) y2[i] = ring0[i * RS + (((s - (rr0 + i - p.halo) + 2) ^ rm) & (kRing - 1))];
 #pragma unroll
             for (int i = 0; i < PR; ++i) {
                 T c0 = acc[i][0], c1 = V::zero();
@@ -463,7 +489,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
 #pragma unroll
                 for (int o = 1; o < S; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                 // lanes without a pixel store to scratch words
-                float* rg = ring0 + i * RS + ((s - (rr0 + i - p.halo)) & (kRing - 1)) * CS + a;
+                float* rg = ring0 + i * RS + (((s - (rr0 + i - p.halo)) ^ rm) & (kRing - 1));
                 const bool inside = (unsigned)col[i] < width[i];
                 if constexpr (HALO) {                            // halo row: the value the band above left
                     const float h = *rg;
@@ -471,6 +497,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
                 }
                 x = inside ? x : 0.f;
                 *(pub[i] ? ex_wr + wr + i * CS : dummy) = x;
+                *(pub[i] ? ey_wr + (odd ? yrow : 0) + i * CS : dummy) = y2[i];
                 *(pub[i] && inside && (!HALO || rr0 + i >= p.halo) ? rg : dummy) = x;
             }
             // off the dependent chain: the pending sums of the next columns, two per column (even and odd kernel rows), so that no
@@ -510,19 +537,22 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
                 __syncwarp();
                 if (t > 0 && lane == 0) mbar_arrive(done_bar + (t & 1));
                 mbar_wait_or_give_up(ready_bar + (t & 1), (t >> 1) & 1, gave_up);
-                if (t >= t_lo && t < t_hi) {                     // warp-uniform
-                    if (t == 0) {
-                        // the first row's first pixel: its right-hand side is otherwise taken one step ahead
+                if (t == 0) {
+                    // what step -1 would have left: the first row's first right-hand side in its pending sum, every row's next one
+                    // in the exchange buffer that step 0 reads
 #pragma unroll
-                        for (int i = 0; i < PR; ++i) {
-                            T rh[NV];
-                            V::template load<AL16>(ring0 + i * RS + sl * NB, rh);
-                            if (rr0 + i == p.halo) {
+                    for (int i = 0; i < PR; ++i) {
+                        if (pub[i]) ey_wr[yrow + i * CS] = ring0[i * RS + (((1 - (rr0 + i - p.halo)) ^ rm) & (kRing - 1))];
+                        if (live && rr0 + i == p.halo) {
+                            float f[NB];
 #pragma unroll
-                                for (int q = 0; q < NV; ++q) acc[i][0] = V::fma(W0[q], rh[q], acc[i][0]);
-                            }
+                            for (int q = 0; q < NB; ++q) f[q] = sl * NB + q < C ? RG[(rr0 + i) * RS + (sl * NB + q) * kChan + rm] : 0.f;
+#pragma unroll
+                            for (int q = 0; q < NV; ++q) acc[i][0] = V::fma(W0[q], V::pick(f, q), acc[i][0]);
                         }
                     }
+                }
+                if (t >= t_lo && t < t_hi) {                     // warp-uniform
 #pragma unroll(UNR)
                     for (int u = 0; u < 8; ++u) {
                         bar_sync(1, nct);                        // every row's pixel of the step before is published
@@ -537,33 +567,33 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         __syncwarp();
         if (lane == 0) mbar_arrive(done_bar + (T_compute & 1));
     } else {
-        // at time t (interval t of the compute warps): store what interval t-1 finished, bring chunk t+2, which interval t+1 waits for
-        if (!p.rot && p.logdet_out != nullptr && blockIdx.x == 0 && warp == p.ncw) warp_logdet(p.w, p.logdet_out, C, HW, K, lane);
-        if (!p.bf16) {
-            copy(0);
-            copy(1);
-            cp_async_mbar_arrive(ready_bar);
+        // At time t (interval t of the compute warps) the storing warps store what interval t-1 finished, the loading warps bring chunk
+        // t+2, which interval t+1 waits for; they hand it over only when the finished chunk has been read, so that neither
+        // side falls more than one interval behind.
+        if (!loader) {
+            if (!p.rot && p.logdet_out != nullptr && blockIdx.x == 0 && warp == p.ncw + p.niow) warp_logdet(p.w, p.logdet_out, C, HW, K, lane);
 #pragma unroll 1
-            for (int t = 0; t <= T_end; ++t) {
-                if (t > 0 && t <= T_compute) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
-                if (t > 0) store(t - 1);
-                if (p.mix_out != nullptr) bar_sync(2, nio);      // the mix reads every channel of a pixel before any is overwritten
-                if (t + 1 < T_compute) {
-                    copy(t + 2);
-                    cp_async_mbar_arrive(ready_bar + ((t + 1) & 1));
-                }
+            for (int t = 1; t <= T_end; ++t) {
+                if (t <= T_compute) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                store(t);
+            }
+        } else if (!p.bf16) {
+#pragma unroll 1
+            for (int t = -2; t + 1 < T_compute; ++t) {
+                if (t > 0) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                copy(t + 2);
+                if (t > 0) mbar_wait_or_give_up(read_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                if (t >= -1) cp_async_mbar_arrive(ready_bar + ((t + 1) & 1));
             }
         } else {
             unsigned pre[4 * BV];
 #pragma unroll 1
-            for (int t = -3; t <= T_end; ++t) {
-                if (t > 0 && t <= T_compute) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
-                if (t > 0) store(t - 1);
-                if (t + 1 < T_compute) {
-                    if (t >= -2) place(pre, t + 2);
-                    if (t >= -1) mbar_arrive(ready_bar + ((t + 1) & 1));
-                    request(pre);
-                }
+            for (int t = -3; t + 1 < T_compute; ++t) {
+                if (t > 0) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                if (t >= -2) place(pre, t + 2);
+                if (t > 0) mbar_wait_or_give_up(read_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                if (t >= -1) mbar_arrive(ready_bar + ((t + 1) & 1));
+                request(pre);
             }
         }
     }

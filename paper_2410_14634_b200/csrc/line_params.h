@@ -19,8 +19,9 @@ struct LineParams {
     int vec;               // W is a multiple of four and every image pointer is aligned to four elements: pieces of four columns
     int bk_warps, bk_parts, bk_per;   // kernel transform: warps per share of the rows, shares, rows per share
     FastDiv div_bk;
-    int ncw, niow;         // compute warps, I/O warps
-    int off_dummy, off_ring, off_a, off_w, off_li;   // float offsets in shared memory
+    int pieces;            // pieces of four columns per I/O thread and chunk
+    int ncw, niow;         // compute warps; loading warps, and as many storing ones
+    int off_dummy, off_y, off_ring, off_a, off_w, off_li;   // float offsets in shared memory
     // the flow step's per-pixel neighbours (see WarpParams): u = V (s x + b) beside x; grad_x = s V^T grad_u on the way in
     const float* mix_V; const float* mix_s; const float* mix_b; float* mix_out; int mix_in;
     float* logdet_out;

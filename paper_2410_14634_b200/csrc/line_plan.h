@@ -15,7 +15,7 @@ namespace invconv {
     X(2, 12, 2, 2, 512, 17, 24) X(2, 16, 2, 2, 384, 25, 32)
 #define INVCONV_LINE_K3(X) \
     X(3, 1, 1, 1, 768, 1, 1) X(3, 2, 1, 1, 768, 2, 2) X(3, 3, 1, 1, 640, 3, 3) X(3, 4, 1, 1, 640, 4, 4) \
-    X(3, 6, 1, 1, 512, 5, 6) X(3, 8, 1, 1, 512, 7, 8) X(3, 12, 1, 1, 256, 9, 12) X(3, 6, 2, 1, 512, 9, 12) X(3, 12, 1, 2, 256, 9, 12) \
+    X(3, 6, 1, 1, 512, 5, 6) X(3, 8, 1, 1, 512, 7, 8) X(3, 12, 1, 1, 384, 9, 12) X(3, 12, 1, 2, 256, 9, 12) \
     X(3, 8, 2, 2, 384, 13, 16) X(3, 6, 4, 4, 384, 17, 24) X(3, 8, 4, 4, 256, 25, 32)
 #define INVCONV_LINE_K5(X) \
     X(5, 1, 1, 1, 640, 1, 1) X(5, 2, 1, 1, 512, 2, 2) X(5, 3, 1, 1, 512, 3, 3) X(5, 4, 1, 1, 384, 4, 4) \
@@ -33,20 +33,16 @@ struct LinePlan {
     bool ok = false;
     int NB = 0, S = 0, PR = 0;
     int HB = 0, nbands = 0, halo = 0, SW = 0;
-    int ncw = 0, niow = 0, grid = 0;
+    int ncw = 0, niow = 0, grid = 0;                  // compute warps; loading warps, and as many storing ones
+    int pieces = 0;
     int bk_warps = 0, bk_parts = 0, bk_per = 0;       // kernel transform: warps per share of the rows, shares, rows per share
-    int off_dummy = 0, off_ring = 0, off_a = 0, off_w = 0, off_li = 0;
+    int off_dummy = 0, off_y = 0, off_ring = 0, off_a = 0, off_w = 0, off_li = 0;
     size_t smem = 0;
     double cycles = 0;      // estimated time of the wavefront
 };
 
 __host__ __device__ constexpr int line_cs(int NB, int S) { return (S * NB + 3) / 4 * 4; }
-// Floats between the rows of a ring: padded so that consecutive rows, whose current pixels are one column apart, fall in
-// different 16-byte banks (row stride minus pixel stride is an odd multiple of 16 bytes modulo 128).
-__host__ __device__ constexpr int line_row_stride(int cols, int CS) { return cols * CS + (CS % 8 == 4 ? 8 : 4); }
-
-// Pieces of four columns that an I/O thread moves per chunk: fewer I/O warps where the weights need the registers.
-__host__ __device__ constexpr int line_pieces(int NB, int S) { return NB * S >= 12 ? 6 : 4; }
+constexpr int kLinePieces = 8;      // pieces of four columns that an I/O thread moves per chunk, at most
 
 inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, int S, int PR, int MAXT, size_t max_smem, int sms, int max_bands = 32)
 {
@@ -62,9 +58,12 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
         pl.halo = nb > 1 ? K - 1 : 0;
         const int HBt = pl.HB + pl.halo;
         pl.ncw = ((HBt + PR - 1) / PR * C * S + 31) / 32;
-        pl.niow = (HBt * C * 2 + 32 * line_pieces(NB, S) - 1) / (32 * line_pieces(NB, S));
-        if ((pl.ncw + pl.niow) * 32 > MAXT) continue;
-        const int threads = (pl.ncw + pl.niow) * 32;
+        // pieces per I/O thread and chunk: few where a step is short, more where the threads are needed for rows
+        for (int want = 3; want <= kLinePieces; want += (want < 4 ? 1 : 2)) {
+        pl.niow = (HBt * C * 2 + 32 * want - 1) / (32 * want);
+        pl.pieces = (HBt * C * 2 + 32 * pl.niow - 1) / (32 * pl.niow);
+        const int threads = (pl.ncw + 2 * pl.niow) * 32;
+        if (threads > MAXT) continue;
         pl.bk_warps = (C * (K * K - 1) + 31) / 32;
         if (pl.bk_warps > pl.ncw) pl.bk_warps = pl.ncw;
         pl.bk_parts = pl.ncw / pl.bk_warps;
@@ -81,7 +80,8 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
         pl.SW = sw;
         int off = up(2 * (HBt + K - 1 + PR) * CS);
         pl.off_dummy = off; off += 32;
-        pl.off_ring = off;  off = up(off + (HBt + PR) * line_row_stride(32, CS));
+        pl.off_y = off;     off = up(off + 2 * (HBt + PR) * CS);
+        pl.off_ring = off;  off = up(off + (HBt + PR) * C * 68);
         pl.off_a = off;     off = up(off + (C | 1) * K * K * CSB);
         pl.off_li = off;    off = up(off + CS * CS);
         pl.off_w = off;     off = up(off + C * C * K * K);
@@ -97,7 +97,10 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
             const int grid = B < o * sms ? B : o * sms;
             const int resident = (grid + sms - 1) / sms, nimg = (B + grid - 1) / grid;
             const double warps = (double)((pl.ncw * resident + 3) / 4);
-            const double step = 150.0 + warps * (1.5 * fma + 35.0);     // fitted to timings of all instances
+            // fitted to timings of all instances; a lone warp on its scheduler issues a multiply-add only every 2.6 cycles
+            double step = 160.0 + 1.5 * fma * (warps < 1.75 ? 1.75 : warps) + 35.0 * warps;
+            const double io = (500.0 + (W % 4 == 0 ? 250.0 : 400.0) * pl.pieces) / 8;
+            if (io > step) step = io;
             const double t = 7000.0 + ((double)(nimg * pl.nbands - 1) * pl.SW + W + pl.HB) * step;
             if (!best.ok || t < best.cycles) {
                 best = pl;
@@ -105,6 +108,7 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
                 best.cycles = t;
                 best.ok = true;
             }
+        }
         }
     }
     return best;
