@@ -224,10 +224,11 @@ struct WarpMix {
 };
 
 // ---------------------------------------------------------------- line wavefront (one thread per row and channel)
-LinePlan line_plan(int B, int C, int H, int W, int k, bool bf16 = false)
+LinePlan line_plan(int B, int C, int H, int W, int k, bool bf16 = false, bool vec = false)
 {
+    // clusters read the rows above a band past the first-level cache, which the single-element copies (vec = false) do not;
     // bfloat16 images are walked in one band only: a band's halo rows come back from the output, where they would be rounded
-    return plan_line(B, C, H, W, k, kMaxDynSmem, sm_count(), bf16 ? 1 : 32);
+    return plan_line(B, C, H, W, k, kMaxDynSmem, sm_count(), bf16 ? 1 : 32, vec && !bf16);
 }
 
 bool line_preferred(int B, int C, int H, int W, int k);
@@ -236,7 +237,10 @@ bool line_preferred(int B, int C, int H, int W, int k);
 int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cudaStream_t st, const WarpMix* mix = nullptr,
                 float* logdet_out = nullptr, bool bf16 = false)
 {
-    const LinePlan pl = line_plan(g.B, g.C, g.H, g.W, g.k, bf16);
+    uintptr_t ptrs = reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out);
+    if (mix && !bwd) ptrs |= reinterpret_cast<uintptr_t>(mix->u_out);
+    const bool vec = g.W % 4 == 0 && (ptrs & (bf16 ? 7 : 15)) == 0;
+    const LinePlan pl = line_plan(g.B, g.C, g.H, g.W, g.k, bf16, vec);
     if (!pl.ok) return INVCONV_UNSUPPORTED;
     LineParams prm = {};
     prm.rhs = rhs; prm.w = w; prm.out = out;
@@ -244,9 +248,8 @@ int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cu
     prm.HB = pl.HB; prm.nbands = pl.nbands; prm.halo = pl.halo; prm.SW = pl.SW;
     prm.div_sw = make_fast_div((unsigned)pl.SW); prm.div_c = make_fast_div((unsigned)g.C); prm.div_nb = make_fast_div((unsigned)pl.nbands);
     prm.rot = bwd ? 1 : 0; prm.bf16 = bf16 ? 1 : 0;
-    uintptr_t ptrs = reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out);
-    if (mix && !bwd) ptrs |= reinterpret_cast<uintptr_t>(mix->u_out);
-    prm.vec = (g.W % 4 == 0 && (ptrs & (bf16 ? 7 : 15)) == 0) ? 1 : 0;
+    prm.vec = vec ? 1 : 0;
+    prm.cluster = pl.cluster;
     prm.ncw = pl.ncw; prm.niow = pl.niow;
     prm.bk_warps = pl.bk_warps; prm.bk_parts = pl.bk_parts; prm.bk_per = pl.bk_per; prm.div_bk = make_fast_div((unsigned)pl.bk_warps);
     prm.pieces = pl.pieces;
@@ -276,7 +279,8 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
                 void* ws, cudaStream_t st, const WarpMix* mix = nullptr, float* logdet_out = nullptr,
                 const LogdetFuse& ld = LogdetFuse{}, bool bf16 = false)
 {
-    if (line_preferred(g.B, g.C, g.H, g.W, g.k) && !(gw && bf16)) {
+    if (line_preferred(g.B, g.C, g.H, g.W, g.k)) {
+        if (gw && bf16) return INVCONV_UNSUPPORTED;    // grad_w takes the fp32 grad_y: the caller converts around the fp32 path
         const int rl = launch_line(bwd, rhs, w, out, g, st, mix, logdet_out, bf16);
         if (rl != INVCONV_UNSUPPORTED) {                // (bfloat16 images of several bands stay with the warp kernel)
             if (rl || !gw) return rl;
@@ -655,16 +659,15 @@ bool line_preferred(int B, int C, int H, int W, int k)
         return C <= 16;
     }
     // WARP shapes.  One lane per row keeps its taps in registers and needs no barrier: it wins while they fit (few channels, k up to
-    // 3) and one warp covers the rows.  Measured, us (WARP / line): C = 3, k = 3: 10.6 / 11.8 at 32x32, 27.8 / 22.0 at 64x64
-    // (batch 32; 28.6 / 31.7 at batch 256), 244 / 215 at 256x256; C = 3, k = 5: 31 / 13 at 32x32; C = 4, k = 3: 13.5 / 12.0 at
-    // 32x32 (14.0 / 17.3 at batch 256); C = 2, k = 5: 10.6 / 11.8 at 32x32, 34.6 / 20.7 at 64x64; C = 1: WARP throughout
-    if (C == 1) return false;
-    if (k == 5) return C >= 3 || H > 32;
+    // 3) and one warp covers the rows.  Measured, us (WARP / line), batch 32: C = 1: 6.4 / 9.5 at 32x32, k = 5 22 / 15 at 64x64;
+    // C = 2: 6.7 / 9.3 at 32x32, 18.6 / 16.6 at 64x64; C = 3: 10.6 / 10.6 at 32x32, 27.7 / 19.9 at 64x64 (28.5 / 41.6 at batch
+    // 256), k = 5 31 / 15 at 32x32; C = 4: 13.4 / 10.3 at 32x32 (14.0 / 14.1 at batch 256), k = 5 36 / 16; images beyond shared
+    // memory: 79 / 69 at C = 1, 244 / 198 at C = 3 (256x256, batch 8)
     if (wp.glb) return true;
+    if (k == 5) return C >= 3 || H > 32;
+    if (C == 1) return false;
     const bool few = B <= sm_count();              // one image per SM: latency counts, not throughput
-    if (C == 2) return H > 32 && W % 4 != 0;
-    if (C == 3) return H > 32 && few;
-    return few && (H > 32 || k == 3);
+    return few && ((H > 32 && H <= 96) || (C == 4 && k == 3));     // 54 / 64 us at 128x128, C = 3
 }
 
 int resolve_path(int B, int C, int H, int W, int k)
@@ -1007,7 +1010,8 @@ size_t invconv_bf16_workspace_bytes(int B, int C, int H, int W, int k)
 {
     if (check_shape(B, C, H, W, k) != INVCONV_OK || B == 0) return 0;
     const size_t need = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k);
-    const bool in_kernel = bf16_in_kernel(B, C, H, W, k, false, false) && bf16_in_kernel(B, C, H, W, k, true, true);
+    const bool in_kernel = bf16_in_kernel(B, C, H, W, k, false, false) && bf16_in_kernel(B, C, H, W, k, true, true) &&
+                           !line_preferred(B, C, H, W, k);
     return need + (in_kernel ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
 }
 
@@ -1090,7 +1094,7 @@ int invconv_forward_bf16(const void* y, const float* w, void* x, int B, int C, i
     if (!y || !w || !x || y == x) return INVCONV_BAD_ARG;
     const bool aligned = ((reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
     const size_t bytes = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k) +
-                         ((aligned && bf16_in_kernel(B, C, H, W, k, false, false)) ? 0 : 2 * up256((size_t)B * C * H * W * sizeof(float)));
+                         ((aligned && bf16_in_kernel(B, C, H, W, k, false, false) && !line_preferred(B, C, H, W, k)) ? 0 : 2 * up256((size_t)B * C * H * W * sizeof(float)));
     StreamScratch sc;
     const int ra = sc.acquire(bytes, as_stream(stream));
     if (ra) return ra;
@@ -1106,7 +1110,7 @@ int invconv_backward_bf16(const void* grad_x, const void* x, const float* w, voi
         return invconv_backward_bf16_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, nullptr, 0, stream);
     const bool aligned = ((reinterpret_cast<uintptr_t>(grad_x) | reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(grad_y)) & 15) == 0;
     const size_t bytes = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k) +
-                         ((aligned && bf16_in_kernel(B, C, H, W, k, true, grad_w != nullptr)) ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
+                         ((aligned && bf16_in_kernel(B, C, H, W, k, true, grad_w != nullptr) && !line_preferred(B, C, H, W, k)) ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
     StreamScratch sc;
     const int ra = sc.acquire(bytes, as_stream(stream));
     if (ra) return ra;

@@ -19,10 +19,12 @@ int launch_line_inst(const invconv::LinePlan& pl, const invconv::LineParams& prm
     cfg.blockDim = dim3((pl.ncw + 2 * pl.niow) * 32);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)pl.cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = pl.cluster > 1 ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, kern, prm) != cudaSuccess) {
         std::fprintf(stderr, "invconv: line launch failed: %s\n", cudaGetErrorString(cudaGetLastError()));
         return INVCONV_CUDA_ERROR;

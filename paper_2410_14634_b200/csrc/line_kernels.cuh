@@ -18,6 +18,10 @@
 // follow one another on one virtual column axis with zero columns between them, so a CTA with several images pays the ramp
 // of the wavefront once.
 //
+// Large images with few of them in a batch are walked by a cluster instead, a band per CTA, all bands at the same time: the band
+// below starts as soon as the bottom rows above have reached global memory (a counter in its shared memory tells; 24
+// columns and the band's height behind).
+//
 // The compute warps share one named barrier per step (a barrier, a shared-memory load and a short dependent sum take about
 // 80 to 110 cycles; an mbarrier that lets a warp's other multiply-adds overlap the wait was measured 60 to 70 cycles
 // slower per step); chunks are handed over between compute and I/O warps through mbarriers.
@@ -119,6 +123,25 @@ struct Vec<NB, true> {
     }
 };
 
+// Add to a counter in a cluster peer's shared memory (after a fence by this thread).
+__device__ __forceinline__ void red_add_cluster(uint32_t remote, unsigned v)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
+// Bounded wait until a counter of this CTA, raised by a cluster peer, reaches `need`; one thread polls, one fence follows (an
+// acquiring poll would pay for it every time).
+__device__ __forceinline__ void wait_count(unsigned* count, unsigned need, volatile int* gave_up)
+{
+    const long long t0 = clock64();
+    for (;;) {
+        unsigned v;
+        asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(count)) : "memory");
+        if (v >= need || *gave_up) break;
+        if (clock64() - t0 > (1ll << 24)) { *gave_up = 1; break; }
+    }
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
+}
+
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
 // The transformed kernel into shared memory: As[(tap*CSB + b)*CA + a], tap = dh*K + dw, CA = C|1, negative for every tap but
@@ -207,7 +230,12 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     extern __shared__ __align__(128) float sm[];
     __shared__ unsigned long long bars[6];             // chunk ready [2], chunk done [2], chunk read for storing [2]
     __shared__ int gave_up_flag;
+    __shared__ unsigned above;                         // cluster: store rounds of the band above, summed over its storing warps
     volatile int* gave_up = &gave_up_flag;
+    // cluster: its CTAs are the bands of one image, all walked at the same time
+    const int crank = p.cluster > 1 ? (int)(blockIdx.x % (unsigned)p.cluster) : 0;
+    const int cid = p.cluster > 1 ? (int)(blockIdx.x / (unsigned)p.cluster) : (int)blockIdx.x;
+    const int ncl = p.cluster > 1 ? (int)(gridDim.x / (unsigned)p.cluster) : (int)gridDim.x;
     const int C = p.C, H = p.H, W = p.W, HW = H * W;
     const int HBt = p.HB + p.halo;
     const int exrow = (HBt + KM + PR) * CS;
@@ -223,9 +251,11 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     float* const dummy = sm + p.off_dummy;             // scratch words for lanes without a pixel
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int NT = blockDim.x, nct = p.ncw * 32;
-    const int nimg = (p.B - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // images blockIdx.x, + gridDim.x, ...
+    const int nimg = (p.B - cid + ncl - 1) / ncl;      // images cid, cid + ncl, ...
     const int nseg = nimg * p.nbands;
-    const int VC = (nseg - 1) * p.SW + W;              // virtual columns
+    // virtual columns; in a cluster the first image starts late enough for the halo rows, which run ahead, to pass their first columns
+    const int lead = p.cluster > 1 ? (K > 9 ? 16 : 8) : 0;
+    const int VC = lead + (nseg - 1) * p.SW + W;
     const int T_compute = (VC + p.HB - 1 + 7) >> 3;    // intervals of eight steps
     const int T_end = ((VC - 1) >> 3) + 1 + ((p.HB - 1 + 7) >> 3);
 
@@ -234,12 +264,17 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         mbar_init(done_bar, p.ncw); mbar_init(done_bar + 1, p.ncw);
         mbar_init(read_bar, p.niow); mbar_init(read_bar + 1, p.niow);
         gave_up_flag = 0;
+        above = 0u;
         fence_mbar_init();
     }
     for (int i = tid; i < 2 * exrow; i += NT) EX[i] = 0.f;
     for (int i = tid; i < 2 * yrow; i += NT) EY[i] = 0.f;          // channels beyond C meet zero weights but must not be NaN
     for (int i = p.off_a + tid; i < p.off_w; i += NT) sm[i] = 0.f;     // As and li
     __syncthreads();
+    if (p.cluster > 1) {                               // the counters exist before the band above adds to them
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
     // everything above touched no global memory; from here on the predecessor kernel's results are needed
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -256,12 +291,13 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
     // per piece, of the chunk moved next: column within its segment, segment, and the element of the segment row's first column
     // (-1: no such row)
     int pcol[BV], pseg[BV], pbase[BV];
+    auto behind = [&](int r) { return r >= -8 && r < 0 ? 0 : r >> 3; };      // chunks behind row 0 when read (halo rows: d columns ahead)
     auto seg_base = [&](int b, int seg) -> int {
         if (seg >= nseg) return -1;
         const int i = p.nbands == 1 ? seg : fast_div(seg, p.div_nb), band = seg - i * p.nbands;
-        const int h = band * p.HB + row[b];
+        const int h = (band + crank) * p.HB + row[b];
         if (h < 0 || h >= H) return -1;
-        return ((int)blockIdx.x + i * (int)gridDim.x) * C * HW + gofs[b] + sgn * band * p.HB * W;
+        return (cid + i * ncl) * C * HW + gofs[b] + sgn * (band + crank) * p.HB * W;
     };
     if (io_warp) {
 #pragma unroll
@@ -271,7 +307,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
             row[b] = ok ? r : -1000000;                // never inside the image
             ring_off[b] = ok ? rr * RS + c * kChan : 0;
             gofs[b] = ok ? c * HW + (p.rot ? HW - 1 - r * W : r * W) : 0;
-            pcol[b] = half4 - (ok ? 8 * ((loader ? r : r + 7) >> 3) : 0);
+            pcol[b] = half4 - lead - (ok ? 8 * (loader ? behind(r) : (r + 7) >> 3) : 0);
             pseg[b] = 0;
             pbase[b] = r < 0 && !loader ? -1 : seg_base(b, 0);
         }
@@ -281,14 +317,14 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         if (nseg > 1)
             while (col >= p.SW) { col -= p.SW; ++seg; base = seg_base(b, seg); }
     };
-    const int safe = (int)blockIdx.x * C * HW;         // an element every load may touch
+    const int safe = cid * C * HW;         // an element every load may touch
     // fp32: asynchronous copies straight into the ring (chunk t), zeros outside the image
     auto copy = [&](int t) {
 #pragma unroll
         for (int b = 0; b < BV; ++b) {
             if (b >= p.pieces) break;                  // uniform
             const bool have = pbase[b] >= 0 && pcol[b] >= 0;
-            const int vc = 8 * (t - (row[b] >> 3)) + half4, left = have ? W - pcol[b] : 0;
+            const int vc = 8 * (t - behind(row[b])) + half4, left = have ? W - pcol[b] : 0;
             const float* g = reinterpret_cast<const float*>(row[b] < 0 ? p.out : p.rhs) + (left > 0 ? pbase[b] + sgn * pcol[b] : safe);
             float* d = RG + ring_off[b];
             if (row[b] > -1000) {
@@ -326,7 +362,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
 #pragma unroll
         for (int b = 0; b < BV; ++b) {
             if (b >= p.pieces) break;
-            const int vc = 8 * (t - (row[b] >> 3)) + half4;
+            const int vc = 8 * (t - behind(row[b])) + half4;
             unsigned u[4];
             if (row[b] <= -1000) continue;
             float* d = RG + ring_off[b];
@@ -441,7 +477,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         unsigned width[PR];
         auto row_width = [&](int i, int bnd) -> unsigned {
             const int r = rr0 + i - p.halo;
-            const bool have = live && rr0 + i < HBt && (r < 0 ? bnd > 0 : bnd * p.HB + r < H);
+            const bool have = live && rr0 + i < HBt && (r < 0 ? bnd + crank > 0 : (bnd + crank) * p.HB + r < H);
             return have ? (unsigned)W : 0u;
         };
 #pragma unroll
@@ -452,7 +488,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         // column within the segment of each row's pixel in the warp's first step; negative before its first column
         int col[PR];
 #pragma unroll
-        for (int i = 0; i < PR; ++i) col[i] = 8 * t_lo - (rr0 + i - p.halo);
+        for (int i = 0; i < PR; ++i) col[i] = 8 * t_lo - lead - (rr0 + i - p.halo);
         bool pub[PR];                                  // this lane publishes the row's pixel
 #pragma unroll
         for (int i = 0; i < PR; ++i) pub[i] = live && sl == 0 && rr0 + i < HBt;
@@ -572,15 +608,30 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         // side falls more than one interval behind.
         if (!loader) {
             if (!p.rot && p.logdet_out != nullptr && blockIdx.x == 0 && warp == p.ncw + p.niow) warp_logdet(p.w, p.logdet_out, C, HW, K, lane);
+            // Tells the band below that a round of stores has reached global memory (its halo rows come from there) -- one round later,
+            // when the fence no longer has to wait for them.
+            auto tell = [&](uint32_t counter) {
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) red_add_cluster(counter, 1u);
+            };
+            const uint32_t below = crank + 1 < p.cluster ? cluster_map_u32(smem_u32(&above), (uint32_t)(crank + 1)) : 0u;
 #pragma unroll 1
             for (int t = 1; t <= T_end; ++t) {
                 if (t <= T_compute) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                if (crank + 1 < p.cluster && t > 1) tell(below);
                 store(t);
             }
+            if (crank + 1 < p.cluster) tell(below);
         } else if (!p.bf16) {
 #pragma unroll 1
             for (int t = -2; t + 1 < T_compute; ++t) {
                 if (t > 0) mbar_wait_or_give_up(done_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
+                if (crank > 0) {                       // chunk t+2 of the bottom rows above has been stored
+                    const unsigned need = (unsigned)(p.niow * min(T_end, t + 3 + ((p.HB - 1 + 7) >> 3)));
+                    if (lane == 0) wait_count(&above, need, gave_up);
+                    __syncwarp();
+                }
                 copy(t + 2);
                 if (t > 0) mbar_wait_or_give_up(read_bar + (t & 1), ((t - 1) >> 1) & 1, gave_up);
                 if (t >= -1) cp_async_mbar_arrive(ready_bar + ((t + 1) & 1));
@@ -598,6 +649,10 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
         }
     }
     __syncthreads();
+    if (p.cluster > 1) {                               // no CTA leaves while the band above may still add to its counter
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
     if (tid == 0 && *gave_up) raise_status(INVCONV_TIMEOUT);
 }
 

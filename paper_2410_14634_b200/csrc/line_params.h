@@ -12,6 +12,7 @@ struct LineParams {
     void* out;             // x or grad_y
     int B, C, H, W;
     int HB, nbands, halo;  // rows per band, bands per image, halo rows (K-1 or 0)
+    int cluster;           // CTAs per image, one band each (1: the bands of an image follow one another in one CTA)
     int SW;                // virtual columns per (image, band)
     FastDiv div_sw, div_c, div_nb;
     int rot;               // 1: transposed solve on the rotated image

@@ -33,6 +33,7 @@ struct LinePlan {
     bool ok = false;
     int NB = 0, S = 0, PR = 0;
     int HB = 0, nbands = 0, halo = 0, SW = 0;
+    int cluster = 1;        // bands of an image walked at the same time by as many CTAs (nbands is then 1)
     int ncw = 0, niow = 0, grid = 0;                  // compute warps; loading warps, and as many storing ones
     int pieces = 0;
     int bk_warps = 0, bk_parts = 0, bk_per = 0;       // kernel transform: warps per share of the rows, shares, rows per share
@@ -44,17 +45,21 @@ struct LinePlan {
 __host__ __device__ constexpr int line_cs(int NB, int S) { return (S * NB + 3) / 4 * 4; }
 constexpr int kLinePieces = 8;      // pieces of four columns that an I/O thread moves per chunk, at most
 
-inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, int S, int PR, int MAXT, size_t max_smem, int sms, int max_bands = 32)
+inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, int S, int PR, int MAXT, size_t max_smem, int sms, int max_bands = 32, bool clusters = false)
 {
     LinePlan best;
     const int CSB = NB * S, CS = line_cs(NB, S);
     auto up = [](int v) { return (v + 31) & ~31; };
+    for (int mode = 0; mode < (clusters ? 2 : 1); ++mode)
     for (int nb = 1; nb <= max_bands && nb <= H; nb = nb + (nb < 8 ? 1 : 4)) {
         LinePlan pl;
         pl.NB = NB; pl.S = S; pl.PR = PR;
         pl.HB = (H + nb - 1) / nb;
         pl.nbands = (H + pl.HB - 1) / pl.HB;
         if (pl.nbands != nb) continue;
+        const bool cl = mode == 1;                     // the bands of an image in a cluster
+        if (cl && nb != 2 && nb != 4 && nb != 8) continue;
+        if (cl) { pl.cluster = nb; pl.nbands = 1; }
         pl.halo = nb > 1 ? K - 1 : 0;
         const int HBt = pl.HB + pl.halo;
         pl.ncw = ((HBt + PR - 1) / PR * C * S + 31) / 32;
@@ -72,7 +77,7 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
         // has stored them (see line_kernels.cuh), chunk alignment lets whole 16-byte pieces move
         int sw = W + K - 1;
         sw = (sw + 3) & ~3;
-        if (nb > 1) {
+        if (nb > 1 && !cl) {
             const int least = 8 * (7 + (pl.HB - 1 + 7) / 8);
             if (sw < least) sw = least;
             sw = (sw + 7) & ~7;
@@ -94,14 +99,17 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
         if (occ > 4) occ = 4;
         const double fma = (double)PR * NB * K * K;
         for (int o = 1; o <= occ; ++o) {
-            const int grid = B < o * sms ? B : o * sms;
-            const int resident = (grid + sms - 1) / sms, nimg = (B + grid - 1) / grid;
+            const int room = o * sms / pl.cluster;     // images in flight
+            if (room < 1) continue;
+            const int images = B < room ? B : room, grid = images * pl.cluster;
+            const int resident = (grid + sms - 1) / sms, nimg = (B + images - 1) / images;
             const double warps = (double)((pl.ncw * resident + 3) / 4);
             // fitted to timings of all instances; a lone warp on its scheduler issues a multiply-add only every 2.6 cycles
             double step = 160.0 + 1.5 * fma * (warps < 1.75 ? 1.75 : warps) + 35.0 * warps;
+            if (nb > 1) step *= 1.15;                  // halo rows
             const double io = (500.0 + (W % 4 == 0 ? 250.0 : 400.0) * pl.pieces) / 8;
             if (io > step) step = io;
-            const double t = 7000.0 + ((double)(nimg * pl.nbands - 1) * pl.SW + W + pl.HB) * step;
+            const double t = 7000.0 + ((double)(nimg * pl.nbands - 1) * pl.SW + W + pl.HB + (pl.cluster - 1) * (pl.HB + 56.0)) * step;
             if (!best.ok || t < best.cycles) {
                 best = pl;
                 best.grid = grid;
@@ -114,13 +122,13 @@ inline LinePlan plan_line_instance(int B, int C, int H, int W, int K, int NB, in
     return best;
 }
 
-inline LinePlan plan_line(int B, int C, int H, int W, int K, size_t max_smem, int sms, int max_bands = 32)
+inline LinePlan plan_line(int B, int C, int H, int W, int K, size_t max_smem, int sms, int max_bands = 32, bool clusters = false)
 {
     LinePlan best;
     if (B < 1) return best;
 #define X(K_, NB_, S_, PR_, MAXT_, CMIN_, CMAX_)                                                                   \
     if (K == K_ && C >= CMIN_ && C <= CMAX_) {                                                                       \
-        const LinePlan pl = plan_line_instance(B, C, H, W, K, NB_, S_, PR_, MAXT_, max_smem, sms, max_bands);            \
+        const LinePlan pl = plan_line_instance(B, C, H, W, K, NB_, S_, PR_, MAXT_, max_smem, sms, max_bands, clusters);            \
         if (pl.ok && (!best.ok || pl.cycles < best.cycles)) best = pl;                                              \
     }
     INVCONV_LINE_ALL(X)
