@@ -31,11 +31,12 @@ struct GradWQuadParams {
     int gst, xst;          // row strides of the staged planes (floats, multiples of 4); x has LP zero columns on its left
     int gfloats, stage;    // floats of the grad_y part and of a whole stage
     int vec;               // rows are 16-byte aligned multiples of 16 bytes
+    int long_rows;         // copied a row per warp, not element by element
     FastDiv div_bands, div_grow, div_gch, div_xch, div_q, div_k;
 };
 
 template <int T, int K>
-__global__ void __launch_bounds__(512) gradw_quad_kernel(const __grid_constant__ GradWQuadParams p)
+__global__ void __launch_bounds__(384, T * T * K <= 32 ? 2 : 1) gradw_quad_kernel(const __grid_constant__ GradWQuadParams p)
 {
     constexpr int LP = (K - 1 + 3) / 4 * 4, NL = 1 + LP / 4;      // zero columns left of the image; 16-byte loads per window
     extern __shared__ __align__(128) float smem[];
@@ -67,6 +68,22 @@ __global__ void __launch_bounds__(512) gradw_quad_kernel(const __grid_constant__
         const int n = fast_div(u, p.div_bands), h0 = (u - n * p.nbands) * RB;
         const float* gsrc = p.gy + ((size_t)n * C + co0) * HW;
         const float* xsrc = p.x + ((size_t)n * C + ci0) * HW;
+        if (p.long_rows) {
+            // long rows of single elements: a row to each warp, its place worked out once (per element that costs 30
+            // against 27 us at 163x3x62x62; but with rows of 9 pixels most of a warp idles, 35 against 24 us at 150x24x9x9)
+            const int grows = nco * RB, rows = grows + nci * xr_rows;
+            for (int q = tid >> 5; q < rows; q += NT >> 5) {
+                const bool isg = q < grows;
+                const int row = isg ? q : q - grows;
+                const int c = isg ? fast_div(row, p.div_gch) : fast_div(row, p.div_xch), r = row - c * (isg ? RB : xr_rows);
+                const int h = h0 + r - (isg ? 0 : K - 1);
+                const bool in = h >= 0 && h < H;
+                const float* src = (isg ? gsrc : xsrc) + (in ? c * HW + h * W : 0);
+                float* dst = base + (isg ? row * p.gst : p.gfloats + row * p.xst + LP);
+                for (int w = lane; w < W; w += 32) cp_async_f32(dst + w, src + w, in);
+            }
+            return;
+        }
         const int ppr = p.vec ? W >> 2 : W;                        // pieces per row
         const int gi = nco * RB * ppr, xi = nci * xr_rows * ppr;
         for (int e = tid; e < gi + xi; e += NT) {

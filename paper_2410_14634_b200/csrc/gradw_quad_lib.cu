@@ -44,6 +44,7 @@ int gradw_quad_launch(const GradWQuadPlan& pl, const float* gy, const float* x, 
     prm.div_grow = make_fast_div((unsigned)(pl.gst / 4));
     prm.div_gch = make_fast_div((unsigned)pl.RB);
     prm.div_xch = make_fast_div((unsigned)(pl.RB + g.k - 1));
+    prm.long_rows = !prm.vec && g.W >= 24;
     prm.div_q = make_fast_div((unsigned)(prm.vec ? g.W / 4 : g.W));
     prm.div_k = make_fast_div((unsigned)g.k);
 #define X(T_, K_) if (pl.T == T_ && g.k == K_) return launch<T_, K_>(pl, prm, dependent, st);

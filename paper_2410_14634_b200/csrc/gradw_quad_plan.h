@@ -46,29 +46,39 @@ inline GradWQuadPlan plan_gradw_quad(int B, int C, int H, int W, int K, size_t m
     pl.threads = 32 * pl.NCO * K * pl.WPT;
     const int groups = pl.tiles * pl.cotiles;
     // shares that fill the SMs once: two CTAs per SM where the sums leave registers for them
-    int want = (T * T * K <= 32 ? 2 : 1) * sms / groups;
+    const bool two = T * T * K <= 32;
+    int want = (two ? 2 : 1) * sms / groups;
     if (want < 1) want = 1;
-    // rows per band: whole images where there are enough of them, bands of at least four rows otherwise
-    int bands = (want + B - 1) / B;
-    if (bands > (H + 3) / 4) bands = (H + 3) / 4;
     pl.gst = (W + 3) & ~3;
     pl.xst = pl.gst + LP;
     if (pl.xst % 32 == 0) pl.xst += 4;
-    for (;; ++bands) {
+    auto fit = [&](int bands) {
         pl.RB = (H + bands - 1) / bands;
         pl.gfloats = pl.NCO * T * pl.RB * pl.gst;
         pl.stage = (pl.gfloats + T * (pl.RB + K - 1) * pl.xst + 31) & ~31;
         pl.smem = sizeof(float) * 2 * (size_t)pl.stage;
         const size_t red = sizeof(float) * (size_t)(pl.threads / 32) * T * T * K;
         if (pl.smem < red) pl.smem = red;
-        if (pl.smem <= max_smem / 2 || pl.RB == 1) break;
+        pl.nbands = (H + pl.RB - 1) / pl.RB;
+        const int units = B * pl.nbands;
+        const int slots = want < units ? want : units, per = (units + slots - 1) / slots;
+        pl.shares = (units + per - 1) / per;           // even shares
+        return (double)((groups * pl.shares + sms - 1) / sms) * per * (pl.RB + K - 1 + (two ? 2 : 8));
+    };
+    // rows per band: the busiest SM stages and walks (CTAs there) x (units of a share) x (rows of a unit with its halo, and a
+    // few rows' worth of waiting, more where no second CTA fills it).  163x3x62x62: 2, 3, 4, 5 bands cost 132, 92, 108, 90 such rows and take 27.1, 22.8, 25.5, 23.9 us;
+    // 32x3x128x128: 10 bands 60 and 17.1 us, 4 to 9 bands 34 and 13.9 us.
+    double best_cost = 1e30;
+    int best_bands = 0;
+    for (int bands = 1; bands <= H; ++bands) {
+        if (bands > (H + 3) / 4 && best_bands) break;
+        const double cost = fit(bands);
+        if (pl.smem > (two ? max_smem / 2 : max_smem) && pl.RB > 1) continue;
+        if (cost < best_cost) { best_cost = cost; best_bands = bands; }
     }
+    if (!best_bands) return pl;
+    fit(best_bands);
     if (pl.smem > max_smem) return pl;
-    pl.nbands = (H + pl.RB - 1) / pl.RB;
-    const int units = B * pl.nbands;
-    pl.shares = want < units ? want : units;
-    const int per = (units + pl.shares - 1) / pl.shares;
-    pl.shares = (units + per - 1) / per;               // even shares
     pl.grid = groups * pl.shares;
     pl.ok = true;
     return pl;
