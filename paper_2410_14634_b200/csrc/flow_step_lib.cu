@@ -353,18 +353,6 @@ int launch_mix(const float* in, const float* V, const float* s, const float* b, 
 
 namespace invconv_internal {
 
-int flow_read_clear_status(int* status_out)
-{
-    int v = 0;
-    if (cudaMemcpyFromSymbol(&v, g_device_status, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
-    if (v != 0) {
-        const int zero = 0;
-        cudaMemcpyToSymbol(g_device_status, &zero, sizeof(int));
-    }
-    *status_out = v;
-    return INVCONV_OK;
-}
-
 int flow_bounds_info(int* info)
 {
 #ifdef INVCONV_DEBUG_BOUNDS

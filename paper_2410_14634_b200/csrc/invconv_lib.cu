@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "invconv.h"
 
@@ -39,7 +40,21 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 }  // namespace
 
+namespace {
+std::vector<invconv_internal::StatusReader>& status_readers()
+{
+    static std::vector<invconv_internal::StatusReader> all;
+    return all;
+}
+}  // namespace
+
 namespace invconv_internal {
+int register_status_reader(StatusReader reader)
+{
+    status_readers().push_back(reader);
+    return 0;
+}
+
 // Called once after every kernel launch of the library.
 int check_launch()
 {
@@ -166,9 +181,31 @@ int launch_gradw_small(const GradWSmallPlan& gs, const float* gy, const float* x
     return invconv_internal::launch_gradw_small_c1(g.k, gs, prm, dep, st);
 }
 
-GradWQuadPlan gradw_quad_plan(int B, int C, int H, int W, int k)
+// The searches for a launch geometry take a microsecond or more, as long as the smallest calls altogether (5.3 against 4.0 us at
+// 2x1x20x20), and a program keeps calling with the same few shapes: each thread keeps the plans of the last ones.
+struct PlanKey {
+    int v[7];
+    bool operator==(const PlanKey& o) const { return std::memcmp(v, o.v, sizeof v) == 0; }
+};
+template <class Plan, class Make>
+const Plan& kept_plan(const PlanKey& key, Make&& make)
 {
-    return plan_gradw_quad(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count());
+    struct Slot { bool set = false; PlanKey key; Plan plan; };
+    thread_local Slot slots[16];
+    unsigned h = 2166136261u;
+    for (int x : key.v) h = (h ^ (unsigned)x) * 16777619u;
+    Slot& s = slots[(h >> 16 ^ h) & 15];
+    if (!s.set || !(s.key == key)) {
+        s.plan = make();
+        s.key = key; s.set = true;
+    }
+    return s.plan;
+}
+
+const GradWQuadPlan& gradw_quad_plan(int B, int C, int H, int W, int k)
+{
+    const int b = B > 0 ? B : 1, sms = sm_count();
+    return kept_plan<GradWQuadPlan>(PlanKey{{b, C, H, W, k, sms, 0}}, [&] { return plan_gradw_quad(b, C, H, W, k, kMaxDynSmem, sms); });
 }
 
 // Fixed-order sum of the shares' partial sums into grad_w.
@@ -224,21 +261,22 @@ struct WarpMix {
 };
 
 // ---------------------------------------------------------------- line wavefront (one thread per row and channel)
-LinePlan line_plan(int B, int C, int H, int W, int k, bool bf16 = false, bool vec = false)
+const LinePlan& line_plan(int B, int C, int H, int W, int k, bool bf16 = false, bool vec = false)
 {
     // clusters read the rows above a band past the first-level cache, which the single-element copies (vec = false) do not;
     // bfloat16 images are walked in one band only: a band's halo rows come back from the output, where they would be rounded
-    return plan_line(B, C, H, W, k, kMaxDynSmem, sm_count(), bf16 ? 1 : 32, vec && !bf16);
+    const int sms = sm_count();
+    return kept_plan<LinePlan>(PlanKey{{B, C, H, W, k, sms, (bf16 ? 1 : 0) + (vec ? 2 : 0)}},
+                               [&] { return plan_line(B, C, H, W, k, kMaxDynSmem, sms, bf16 ? 1 : 32, vec && !bf16); });
 }
 
-bool line_preferred(int B, int C, int H, int W, int k);
+bool line_preferred(int B, int C, int H, int W, int k, bool bwd, bool bf16 = false);
 
 // The solve through the line wavefront; INVCONV_UNSUPPORTED where it has no plan.
 int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cudaStream_t st, const WarpMix* mix = nullptr,
                 float* logdet_out = nullptr, bool bf16 = false)
 {
-    uintptr_t ptrs = reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out);
-    if (mix && !bwd) ptrs |= reinterpret_cast<uintptr_t>(mix->u_out);
+    const uintptr_t ptrs = reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out);
     const bool vec = g.W % 4 == 0 && (ptrs & (bf16 ? 7 : 15)) == 0;
     const LinePlan pl = line_plan(g.B, g.C, g.H, g.W, g.k, bf16, vec);
     if (!pl.ok) return INVCONV_UNSUPPORTED;
@@ -255,8 +293,7 @@ int launch_line(bool bwd, const void* rhs, const float* w, void* out, Geom g, cu
     prm.pieces = pl.pieces;
     prm.off_dummy = pl.off_dummy; prm.off_y = pl.off_y; prm.off_ring = pl.off_ring; prm.off_a = pl.off_a; prm.off_w = pl.off_w; prm.off_li = pl.off_li;
     if (mix) {
-        prm.mix_V = mix->V; prm.mix_s = mix->s; prm.mix_b = mix->b;
-        prm.mix_out = bwd ? nullptr : mix->u_out;
+        prm.mix_V = mix->V; prm.mix_s = mix->s;
         prm.mix_in = (bwd && mix->grad_in) ? 1 : 0;
     }
     prm.logdet_out = bwd ? nullptr : logdet_out;
@@ -279,7 +316,7 @@ int launch_warp(bool bwd, const float* rhs, const float* w, float* out, const fl
                 void* ws, cudaStream_t st, const WarpMix* mix = nullptr, float* logdet_out = nullptr,
                 const LogdetFuse& ld = LogdetFuse{}, bool bf16 = false)
 {
-    if (line_preferred(g.B, g.C, g.H, g.W, g.k)) {
+    if (line_preferred(g.B, g.C, g.H, g.W, g.k, bwd, bf16)) {
         if (gw && bf16) return INVCONV_UNSUPPORTED;    // grad_w takes the fp32 grad_y: the caller converts around the fp32 path
         const int rl = launch_line(bwd, rhs, w, out, g, st, mix, logdet_out, bf16);
         if (rl != INVCONV_UNSUPPORTED) {                // (bfloat16 images of several bands stay with the warp kernel)
@@ -455,22 +492,35 @@ GradWTensorPlan gradw_tensor_plan(int B, int C, int H, int W, int k)
     return plan_gradw_tensor(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count());
 }
 
-// The team family: a cluster or CTA per image (team_kernels.cuh), or the line wavefront where that has a plan.
+// The tensor-core wavefront with three-term products: any channel count and image alignment, fp32 accuracy.
+TensorPlan tensor3_plan(int B, int C, int H, int W, int k)
+{
+    if (C <= 4 || team_solve_smem(C, k) > kMaxDynSmem) return TensorPlan{};
+    return plan_tensor(B > 0 ? B : 1, C, H, W, k, kMaxDynSmem, sm_count(), true);
+}
+
+// The team family: a cluster or CTA per image (team_kernels.cuh), or the line wavefront or the three-term tensor-core wavefront
+// where those have a plan.
 bool team_serves(int B, int C, int H, int W, int k)
 {
-    return team_plan(B, C, H, W, k).ok || line_plan(B > 0 ? B : 1, C, H, W, k).ok;
+    return team_plan(B, C, H, W, k).ok || line_plan(B > 0 ? B : 1, C, H, W, k).ok || tensor3_plan(B, C, H, W, k).ok;
 }
 
 // Workspace of the team family: control words, transformed kernel, C*C floats, then the partial sums of
 // grad_w -- one set per batch share of whichever correlation kernel runs (the tcgen05 one included).
+size_t team_wop_offset(int B, int C, int H, int W, int k)      // ... then the tensor-core operands
+{
+    const size_t na = sizeof(float) * (size_t)k * k * C * C;
+    const GradWTensorPlan gt = gradw_tensor_plan(B, C, H, W, k);
+    const int shares = std::max(gradw_quad_plan(B, C, H, W, k).shares, gt.ok ? gt.S : 0);
+    return (INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)C * C + na * shares + 255) & ~(size_t)255;
+}
+
 size_t team_workspace_bytes(int B, int C, int H, int W, int k)
 {
     if (!team_serves(B, C, H, W, k)) return 0;
-    const size_t na = sizeof(float) * (size_t)k * k * C * C;
-    const GradWTensorPlan gt = gradw_tensor_plan(B, C, H, W, k);
-    int shares = gradw_quad_plan(B, C, H, W, k).shares;
-    if (gt.ok && gt.S > shares) shares = gt.S;
-    return INVCONV_WS_CONTROL_BYTES + na + sizeof(float) * (size_t)C * C + na * shares;
+    const TensorPlan t3 = tensor3_plan(B, C, H, W, k);
+    return team_wop_offset(B, C, H, W, k) + (t3.ok ? t3.wop_bytes : 0);
 }
 
 // grad_w in fp32; the partial sums live behind the transformed kernel in the workspace.
@@ -533,19 +583,41 @@ int launch_pixel_inst(const TeamPlan& pl, const TeamParams& prm, cudaStream_t st
     return check_launch();
 }
 
+// Whether the three-term tensor-core wavefront runs in place of the team kernels.  Its step takes about 1.3 us, and the kernel's
+// operands are packed anew in each call; it is behind where the contraction is mostly padding and few team steps follow each other:
+// 4x18x7x9, k = 3: 31 against 24 us; 256x24x4x4: 23 against 18 us.  But 256x18x8x8: 31 against 42, 64x96x8x8: 49 against 84,
+// 256x96x12x12: 192 against 900, 64x22x6x6 with k = 5: 31 against 53 us.  Up to 16 channels: 208x14x20x14: 53 against 78,
+// 41x16x17x9: 43 against 33 us.
+bool tensor3_preferred(const Geom& g)
+{
+    const int n = g.H * g.W;
+    if (g.C <= 16) return n > 324 || (g.k == 5 && n >= 280) || g.B > sm_count();
+    if (g.C <= 24 && n <= 16) return false;
+    if (g.C <= 24 && n <= (g.W % 4 ? 64 : 96) && g.k <= 3 && g.B <= sm_count()) return false;
+    return tensor3_plan(g.B, g.C, g.H, g.W, g.k).ok;
+}
+
 // Transposed or plain solve through the team family; the transformed kernel goes to the workspace.
-int launch_team(bool bwd, const float* rhs, const float* w, float* out, Geom g, void* ws, cudaStream_t st, float* logdet_out = nullptr)
+// `three`: the three-term tensor-core wavefront may run in its place (the workspace is the team family's).
+int launch_team(bool bwd, const float* rhs, const float* w, float* out, Geom g, void* ws, cudaStream_t st, float* logdet_out = nullptr,
+                bool three = false)
 {
     const TeamPlan pl = team_plan(g.B, g.C, g.H, g.W, g.k);
     const bool variant = opt(INVCONV_OPT_TEAM_VARIANT) == 1 || opt(INVCONV_OPT_TEAM_VARIANT) == 2;
-    if ((!pl.ok && !variant) || line_preferred(g.B, g.C, g.H, g.W, g.k)) {
+    if ((!pl.ok && !variant) || line_preferred(g.B, g.C, g.H, g.W, g.k, bwd)) {
         const int rl = launch_line(bwd, rhs, w, out, g, st, nullptr, logdet_out);
         if (rl != INVCONV_UNSUPPORTED) return rl;
+    }
+    if (three && opt(INVCONV_OPT_TEAM_VARIANT) == 0 && (!pl.ok || (g_forced_path.load() == INVCONV_PATH_AUTO && tensor3_preferred(g)))) {
+        const TensorPlan t3 = tensor3_plan(g.B, g.C, g.H, g.W, g.k);
+        unsigned char* wop = static_cast<unsigned char*>(ws) + team_wop_offset(g.B, g.C, g.H, g.W, g.k);
+        const int r3 = t3.ok ? invconv_internal::tensor_launch(t3, bwd, rhs, w, out, g, nullptr, wop, st, logdet_out) : (int)INVCONV_UNSUPPORTED;
+        if (r3 != INVCONV_UNSUPPORTED) return r3;
     }
     if (!pl.ok) return INVCONV_UNSUPPORTED;
     float* A = reinterpret_cast<float*>(static_cast<char*>(ws) + INVCONV_WS_CONTROL_BYTES);
     {
-        if (team_solve_launch(bwd, w, A, g.C, g.k, nullptr, 0, 0u, logdet_out, g.H * g.W, st) != cudaSuccess) {
+        if (team_solve_launch(bwd, w, A, g.C, g.k, nullptr, 0, 0u, g.C, false, logdet_out, g.H * g.W, st) != cudaSuccess) {
             cudaGetLastError();
             return INVCONV_CUDA_ERROR;
         }
@@ -644,7 +716,7 @@ int auto_path(int B, int C, int H, int W, int k)
 
 // Whether the line wavefront runs in place of the family that the shape belongs to (INVCONV_OPT_LINE overrides; a forced family
 // runs its own kernels).
-bool line_preferred(int B, int C, int H, int W, int k)
+bool line_preferred(int B, int C, int H, int W, int k, bool bwd, bool bf16)
 {
     const int knob = opt(INVCONV_OPT_LINE);
     if (knob == 0 || B < 1) return false;
@@ -652,22 +724,37 @@ bool line_preferred(int B, int C, int H, int W, int k)
     if (!pl.ok) return false;
     if (knob == 1) return true;
     if (g_forced_path.load() != INVCONV_PATH_AUTO) return false;
-    const WarpPlan wp = plan_warp(B, C, H, W, k, true);
-    if (!wp.ok) {
-        // TENSOR and TEAM shapes: measured (16x16, k = 3, batch 64) 14.5 against 38 us at C = 12, 16.5 against 43 us at C = 16, but
-        // 95 against 60 us at C = 24, where a CTA's registers no longer hold a band of useful height
-        return C <= 16;
-    }
-    // WARP shapes.  One lane per row keeps its taps in registers and needs no barrier: it wins while they fit (few channels, k up to
-    // 3) and one warp covers the rows.  Measured, us (WARP / line), batch 32: C = 1: 6.4 / 9.5 at 32x32, k = 5 22 / 15 at 64x64;
-    // C = 2: 6.7 / 9.3 at 32x32, 18.6 / 16.6 at 64x64; C = 3: 10.6 / 10.6 at 32x32, 27.7 / 19.9 at 64x64 (28.5 / 41.6 at batch
-    // 256), k = 5 31 / 15 at 32x32; C = 4: 13.4 / 10.3 at 32x32 (14.0 / 14.1 at batch 256), k = 5 36 / 16; images beyond shared
-    // memory: 79 / 69 at C = 1, 244 / 198 at C = 3 (256x256, batch 8)
-    if (wp.glb) return true;
-    if (k == 5) return C >= 3 || H > 32;
-    if (C == 1) return false;
+    const WarpPlan wp = plan_warp(B, C, H, W, k, bwd);
     const bool few = B <= sm_count();              // one image per SM: latency counts, not throughput
-    return few && ((H > 32 && H <= 96) || (C == 4 && k == 3));     // 54 / 64 us at 128x128, C = 3
+    const int n = H * W;
+    if (!wp.ok) {
+        // TEAM and TENSOR shapes.  Up to 12 channels an image's rows are one band of threads, or a second band costs less than the
+        // other families do (10x22x22 with k = 5: 83 against 87 us); above that each further band repeats the whole walk, with fewer
+        // registers per tap (us, line / other, k = 3): one band 13.9 / 24.8 at 16x9x9, 18.0 / 26.9 at 22x8x8; two 62 / 77 at
+        // 16x25x25, 43 / 33 at 16x17x9; more 98 / 85 at 16x28x28, 87 / 43 at 20x13x13; with k = 5 115 / 30 at 16x9x8
+        const int bands = pl.nbands * pl.cluster;
+        if (bands == 1) return C <= 16 || (C <= 24 && few);
+        if (k == 5) return C <= 8 || (C <= 12 && n >= 400);
+        return C <= 12 || (C <= 16 && bands == 2 && few && 2 * B <= sm_count() && n > 256);
+    }
+    // WARP shapes.  That family keeps an image and a row's taps in one warp and needs no barrier: it wins for small images, few
+    // channels and many images; but its copies are 16 bytes wide only if the image is a multiple of that, and rows beyond shared
+    // memory or k = 5 slow it down.  us, WARP / line, forward, batch in brackets:
+    //   image off 16 bytes [17]: 23.5 / 11.4 at 3x29x29, [8] 16.7 / 9.8 at 3x17x17, [3] 19.1 / 14.7 at 1x49x49; 5.0 / 7.4 at 1x21x21
+    //   beyond shared memory: [49] 1.6 times at 3x196x196; but 1x222x222 fits in the forward direction, [11] 52 / 73
+    //   k = 5: [11] 2.4 times at 4x28x28; C = 2: 1.7 to 2.5 times above 32 rows, C = 1: [6] 1.4 times at 64x64
+    //   few images, C = 3: [7] 1.4 times at 44x44, but [204] 0.6 times; 28x28 0.9, 130x130 0.7; C = 4: [8] 1.7 times at 43x43
+    const size_t img = (size_t)C * n;
+    // (bfloat16 images stay in one band: 182 against 127 us at 2x228x159)
+    if (wp.glb) return !(bf16 && !bwd && C <= 2 && img % 4 == 0);
+    if (bf16 && img % 4 != 0) return true;
+    const bool own = bf16 && bwd && img % 8 == 0;  // the WARP kernel takes bfloat16 images and grad_w in one launch
+    if (k == 5) return C >= 3 || (H > 32 && !(C == 1 && img % 4 == 0 && (own || (bwd && W % 4 != 0)))) || (C == 2 && img % 4 != 0);
+    if (img % 4 != 0) return C >= 3 || (C == 2 ? H > 32 || (n > 400 && few) : H > 36 && few);
+    if (C <= 2) return false;
+    if (W % 4 != 0 && H > 80 && (B > 64 || (bf16 && (!bwd || k == 2)))) return false;
+    if (C == 3) return few && H > (own ? 64 : 32) && H <= 96;
+    return few && H <= 96 && (H > 32 || (k == 3 && !(bf16 && img % 8 == 0)));
 }
 
 int resolve_path(int B, int C, int H, int W, int k)
@@ -714,18 +801,9 @@ int launch_forward(int path, const float* y, const float* w, float* x, Geom g,
     case INVCONV_PATH_WARP:
         return launch_warp(false, y, w, x, nullptr, nullptr, g, ws, st, nullptr, logdet_out);
     case INVCONV_PATH_TEAM:
-        return launch_team(false, y, w, x, g, ws, st, logdet_out);
+        return launch_team(false, y, w, x, g, ws, st, logdet_out, true);
     case INVCONV_PATH_TENSOR: {
-        // buffers off a 16-byte boundary cannot use the bulk copies of the tensor family: the team family serves
-        // them from the same workspace (its layout is a prefix of the tensor family's)
-        const bool aligned = ((reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
-        if (line_preferred(g.B, g.C, g.H, g.W, g.k)) return launch_team(false, y, w, x, g, ws, st, logdet_out);
-        if (!aligned && g_forced_path.load() == INVCONV_PATH_AUTO) {
-            if (team_serves(g.B, g.C, g.H, g.W, g.k)) return launch_team(false, y, w, x, g, ws, st, logdet_out);
-            generic_wavefront_kernel<false><<<g.B, 256, 0, st>>>(y, w, x, g);      // neither family takes them: the generic one does
-            const int rc = check_launch();
-            return rc ? rc : separate_logdet();
-        }
+        if (line_preferred(g.B, g.C, g.H, g.W, g.k, false)) return launch_team(false, y, w, x, g, ws, st, logdet_out);
         return launch_tensor(false, y, w, x, g, ws, st, logdet_out);
     }
     default:
@@ -757,27 +835,15 @@ int launch_backward(int path, const float* gx, const float* x, const float* w, f
         return launch_warp(true, gx, w, gy, x, gw, g, ws, st, nullptr, nullptr, ld);
     case INVCONV_PATH_TEAM: {
         if (g.B > 0) {
-            const int rc = launch_team(true, gx, w, gy, g, ws, st);
+            const int rc = launch_team(true, gx, w, gy, g, ws, st, nullptr, true);
             if (rc) return rc;
         }
         return gw ? launch_gradw_many(path, gy, x, gw, g, ws, st, ld) : INVCONV_OK;
     }
     case INVCONV_PATH_TENSOR: {
         if (g.B > 0) {
-            const bool aligned = ((reinterpret_cast<uintptr_t>(gx) | reinterpret_cast<uintptr_t>(gy)) & 15) == 0;
-            int rc;
-            if (line_preferred(g.B, g.C, g.H, g.W, g.k)) {
-                rc = launch_team(true, gx, w, gy, g, ws, st);
-            } else if (!aligned && g_forced_path.load() == INVCONV_PATH_AUTO) {
-                if (team_serves(g.B, g.C, g.H, g.W, g.k)) {
-                    rc = launch_team(true, gx, w, gy, g, ws, st);
-                } else {
-                    generic_wavefront_kernel<true><<<g.B, 256, 0, st>>>(gx, w, gy, g);
-                    rc = check_launch();
-                }
-            } else {
-                rc = launch_tensor(true, gx, w, gy, g, ws, st);
-            }
+            const int rc = line_preferred(g.B, g.C, g.H, g.W, g.k, true) ? launch_team(true, gx, w, gy, g, ws, st)
+                                                                   : launch_tensor(true, gx, w, gy, g, ws, st);
             if (rc) return rc;
         }
         return gw ? launch_gradw_many(path, gy, x, gw, g, ws, st, ld) : INVCONV_OK;
@@ -910,7 +976,8 @@ namespace invconv_internal {
 int warp_step_forward(const float* y, const float* w, const float* s, const float* b, const float* V, float* x, float* u,
                       Geom g, void* ws, cudaStream_t st)
 {
-    if (resolve_path(g.B, g.C, g.H, g.W, g.k) != INVCONV_PATH_WARP) return INVCONV_UNSUPPORTED;
+    // (the line wavefront's storing warps fall behind with the mixing in them: 491 us where the solve alone takes 165, at 3x211x211)
+    if (resolve_path(g.B, g.C, g.H, g.W, g.k) != INVCONV_PATH_WARP || line_preferred(g.B, g.C, g.H, g.W, g.k, false)) return INVCONV_UNSUPPORTED;
     WarpMix mix;
     mix.V = V; mix.s = s; mix.b = b; mix.u_out = u;
     return launch_warp(false, y, w, x, nullptr, nullptr, g, ws, st, &mix);
@@ -924,7 +991,7 @@ int warp_step_backward(const float* grad_u, const float* x, const float* w, cons
     mix.V = V; mix.s = s; mix.grad_in = true;
     if (path != INVCONV_PATH_WARP) {
         // the line wavefront takes the neighbours with the kernel: its right-hand side enters through A_0 diag(s) V^T
-        if (path == INVCONV_PATH_GENERIC || !line_preferred(g.B, g.C, g.H, g.W, g.k)) return INVCONV_UNSUPPORTED;
+        if (path == INVCONV_PATH_GENERIC || !line_preferred(g.B, g.C, g.H, g.W, g.k, true)) return INVCONV_UNSUPPORTED;
         const int rc = launch_line(true, grad_u, w, grad_y, g, st, &mix);
         return rc ? rc : launch_gradw_many(path, grad_y, x, grad_w, g, ws, st, LogdetFuse{});
     }
@@ -1011,7 +1078,7 @@ size_t invconv_bf16_workspace_bytes(int B, int C, int H, int W, int k)
     if (check_shape(B, C, H, W, k) != INVCONV_OK || B == 0) return 0;
     const size_t need = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k);
     const bool in_kernel = bf16_in_kernel(B, C, H, W, k, false, false) && bf16_in_kernel(B, C, H, W, k, true, true) &&
-                           !line_preferred(B, C, H, W, k);
+                           !line_preferred(B, C, H, W, k, false, true) && !line_preferred(B, C, H, W, k, true, true);
     return need + (in_kernel ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
 }
 
@@ -1032,7 +1099,7 @@ int invconv_forward_bf16_ws(const void* y, const float* w, void* x, int B, int C
                                    nullptr, nullptr, LogdetFuse{}, true);
         if (rw != INVCONV_UNSUPPORTED) return rw;
     }
-    if (path != INVCONV_PATH_WARP && line_preferred(B, C, H, W, k)) {
+    if (path != INVCONV_PATH_WARP && line_preferred(B, C, H, W, k, false, true)) {
         const int rl = launch_line(false, y, w, x, g, st, nullptr, nullptr, true);
         if (rl != INVCONV_UNSUPPORTED) return rl;
     }
@@ -1070,7 +1137,7 @@ int invconv_backward_bf16_ws(const void* grad_x, const void* x, const float* w, 
                                    static_cast<const float*>(x), grad_w, g, workspace, st, nullptr, nullptr, LogdetFuse{}, true);
         if (rw != INVCONV_UNSUPPORTED) return rw;
     }
-    if (path != INVCONV_PATH_WARP && !grad_w && line_preferred(B, C, H, W, k)) {
+    if (path != INVCONV_PATH_WARP && !grad_w && line_preferred(B, C, H, W, k, true, true)) {
         const int rl = launch_line(true, grad_x, w, grad_y, g, st, nullptr, nullptr, true);
         if (rl != INVCONV_UNSUPPORTED) return rl;
     }
@@ -1094,7 +1161,7 @@ int invconv_forward_bf16(const void* y, const float* w, void* x, int B, int C, i
     if (!y || !w || !x || y == x) return INVCONV_BAD_ARG;
     const bool aligned = ((reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
     const size_t bytes = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k) +
-                         ((aligned && bf16_in_kernel(B, C, H, W, k, false, false) && !line_preferred(B, C, H, W, k)) ? 0 : 2 * up256((size_t)B * C * H * W * sizeof(float)));
+                         ((aligned && bf16_in_kernel(B, C, H, W, k, false, false) && !line_preferred(B, C, H, W, k, false, true)) ? 0 : 2 * up256((size_t)B * C * H * W * sizeof(float)));
     StreamScratch sc;
     const int ra = sc.acquire(bytes, as_stream(stream));
     if (ra) return ra;
@@ -1110,7 +1177,7 @@ int invconv_backward_bf16(const void* grad_x, const void* x, const float* w, voi
         return invconv_backward_bf16_ws(grad_x, x, w, grad_y, grad_w, B, C, H, W, k, nullptr, 0, stream);
     const bool aligned = ((reinterpret_cast<uintptr_t>(grad_x) | reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(grad_y)) & 15) == 0;
     const size_t bytes = bf16_ws_need(resolve_path(B, C, H, W, k), B, C, H, W, k) +
-                         ((aligned && bf16_in_kernel(B, C, H, W, k, true, grad_w != nullptr) && !line_preferred(B, C, H, W, k)) ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
+                         ((aligned && bf16_in_kernel(B, C, H, W, k, true, grad_w != nullptr) && !line_preferred(B, C, H, W, k, true, true)) ? 0 : 3 * up256((size_t)B * C * H * W * sizeof(float)));
     StreamScratch sc;
     const int ra = sc.acquire(bytes, as_stream(stream));
     if (ra) return ra;
@@ -1404,17 +1471,13 @@ int invconv_get_status(void* stream, int* device_status_out)
 {
     if (!device_status_out) return INVCONV_BAD_ARG;
     if (cudaStreamSynchronize(as_stream(stream)) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
-    int v = 0, vt = 0;
-    if (cudaMemcpyFromSymbol(&v, g_device_status, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
-    if (v != 0) {
-        const int zero = 0;
-        cudaMemcpyToSymbol(g_device_status, &zero, sizeof(int));
+    int worst = 0;
+    for (const invconv_internal::StatusReader reader : status_readers()) {
+        int v = 0;
+        if (reader(&v) != INVCONV_OK) return INVCONV_CUDA_ERROR;
+        worst = std::max(worst, v);
     }
-    if (invconv_internal::tensor_read_clear_status(&vt) != INVCONV_OK) return INVCONV_CUDA_ERROR;
-    int vf = 0;
-    if (invconv_internal::flow_read_clear_status(&vf) != INVCONV_OK) return INVCONV_CUDA_ERROR;
-    if (vf > vt) vt = vf;
-    *device_status_out = v > vt ? v : vt;
+    *device_status_out = worst;
     return INVCONV_OK;
 }
 

@@ -14,6 +14,7 @@
 namespace invconv {
 struct LineParams;
 struct WarpParams;
+struct TensorParams;
 struct GradWSmallPlan;
 struct GradWSmallParams;
 }  // namespace invconv
@@ -21,6 +22,25 @@ struct GradWSmallParams;
 namespace invconv_internal {
 
 constexpr size_t kMaxDynSmem = 226 * 1024;   // 227 KiB per CTA minus the kernels' static shared memory
+
+// Every translation unit has its own copy of the device status word (common.cuh); each registers the function that reads and clears
+// its copy on the current device, and invconv_get_status asks all of them.
+using StatusReader = int (*)(int*);
+int register_status_reader(StatusReader reader);
+namespace {
+int read_clear_status(int* status_out)
+{
+    int v = 0;
+    if (cudaMemcpyFromSymbol(&v, invconv::g_device_status, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
+    if (v != 0) {
+        const int zero = 0;
+        cudaMemcpyToSymbol(invconv::g_device_status, &zero, sizeof(int));
+    }
+    *status_out = v;
+    return INVCONV_OK;
+}
+[[maybe_unused]] const int status_reader_registered = register_status_reader(&read_clear_status);
+}  // namespace
 
 // Counts the launch and turns cudaGetLastError into a status code.
 int check_launch();
@@ -53,8 +73,8 @@ int warp_step_backward(const float* grad_u, const float* x, const float* w, cons
 // tensor_lib.cu: the tcgen05 wavefront (kernel transform into A, operand packing into wop, solve).
 int tensor_launch(const invconv::TensorPlan& pl, bool bwd, const float* rhs, const float* w, float* out,
                   invconv::Geom g, float* A, unsigned char* wop, cudaStream_t st, float* logdet_out = nullptr);
-int tensor_read_clear_status(int* status_out);
-int flow_read_clear_status(int* status_out);              // flow_step_lib.cu's copy of the status word
+// tensor3_lib.cu: the same wavefront with three-term products.
+int tensor3_launch(const invconv::TensorPlan& pl, const invconv::TensorParams& prm, int k, cudaStream_t st);
 int tensor_bounds_info(int* info);                        // debug-bounds build: first violation and count (both units)
 int flow_bounds_info(int* info);
 int tensor_selftest_bounds(cudaStream_t st);

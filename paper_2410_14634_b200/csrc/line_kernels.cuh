@@ -377,12 +377,6 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
             }
         }
     };
-    // u = V (s x + b) of the flow step for one channel of one pixel
-    auto mixed = [&](const float* px, int c) -> float {
-        float u = 0.f;
-        for (int m = 0; m < C; ++m) u = fmaf(__ldg(p.mix_V + c * C + m), fmaf(__ldg(p.mix_s + m), px[m * kChan], __ldg(p.mix_b + m)), u);
-        return u;
-    };
     auto hand_back = [&](int t) {                      // the finished chunk has been read
         __syncwarp();
         if (lane == 0) mbar_arrive(read_bar + (t & 1));
@@ -397,7 +391,7 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
             const int vc = 8 * (t - 1 - ((row[b0 + q] + 7) >> 3)) + half4;
             f[q] = *reinterpret_cast<const float4*>(RG + ring_off[b0 + q] + (((vc ^ rm) & (kRing - 1)) & ~3));      // memory order
         }
-        if (p.mix_out == nullptr && b0 + 4 >= p.pieces) hand_back(t);
+        if (b0 + 4 >= p.pieces) hand_back(t);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int b = b0 + q;
@@ -426,13 +420,8 @@ __global__ void __launch_bounds__(MAXT, 1) line_wavefront_kernel(const __grid_co
                     }
                 }
             }
-            if (p.mix_out != nullptr) {                  // forward only: slots are virtual columns
-                const int rr = row[b] + p.halo, c = (ring_off[q] - rr * RS) / kChan, vc = 8 * (t - 1 - ((row[b] + 7) >> 3)) + half4;
-                for (int j = 0; j < nv; ++j) p.mix_out[i + j] = mixed(RG + rr * RS + ((vc + j) & (kRing - 1)), c);
-            }
         }
         }
-        if (p.mix_out != nullptr) hand_back(t);
     };
     if (!io_warp) {
         {

@@ -23,8 +23,8 @@ struct LineParams {
     int pieces;            // pieces of four columns per I/O thread and chunk
     int ncw, niow;         // compute warps; loading warps, and as many storing ones
     int off_dummy, off_y, off_ring, off_a, off_w, off_li;   // float offsets in shared memory
-    // the flow step's per-pixel neighbours (see WarpParams): u = V (s x + b) beside x; grad_x = s V^T grad_u on the way in
-    const float* mix_V; const float* mix_s; const float* mix_b; float* mix_out; int mix_in;
+    // the flow step's per-pixel neighbours (see WarpParams) on the way in: grad_x = s V^T grad_u
+    const float* mix_V; const float* mix_s; int mix_in;
     float* logdet_out;
 };
 

@@ -60,9 +60,29 @@ inline size_t team_solve_smem(int C, int K)
     return sizeof(float) * ((size_t)C * (32 * team_solve_ns(C) + 1) + ((C + 3) & ~3) + (size_t)C * nc + (size_t)C * (nc | 1));
 }
 
+// Value v of input channel j (of a chunk's eight) and operand row `row` in the operand form of the tensor-core kernels:
+// planes of 16-byte rows, two-term (tf32 hi in planes 0, 1; bf16 remainder; bf16 value) or three-term (bf16 terms w0, w1, w0, w2).
+__device__ __forceinline__ void pack_operand(unsigned char* blk, int rows, int row, int j, float v, bool three)
+{
+    if (three) {
+        const __nv_bfloat16 a = __float2bfloat16_rn(v);
+        const float r = v - __bfloat162float(a);
+        const __nv_bfloat16 b = __float2bfloat16_rn(r);
+        *reinterpret_cast<__nv_bfloat16*>(blk + (size_t)row * 16 + j * 2) = a;
+        *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)rows + row) * 16 + j * 2) = b;
+        *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)2 * rows + row) * 16 + j * 2) = a;
+        *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)3 * rows + row) * 16 + j * 2) = __float2bfloat16_rn(r - __bfloat162float(b));
+    } else {
+        const float hi = tf32_hi(v);
+        *reinterpret_cast<float*>(blk + ((size_t)(j >> 2) * rows + row) * 16 + (j & 3) * 4) = hi;
+        *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)2 * rows + row) * 16 + j * 2) = __float2bfloat16_rn(v - hi);
+        *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)3 * rows + row) * 16 + j * 2) = __float2bfloat16_rn(v);
+    }
+}
+
 template <bool BWD, int NS>
 __global__ void __launch_bounds__(512) team_solve_kernel(const float* __restrict__ w, float* __restrict__ A, int C, int K,
-                                                         unsigned char* __restrict__ wop, int NCH, unsigned wbytes,
+                                                         unsigned char* __restrict__ wop, int NCH, unsigned wbytes, int CP_, int three,
                                                          float* __restrict__ logdet_out, int HW)
 {
     extern __shared__ __align__(128) float sm[];
@@ -73,14 +93,24 @@ __global__ void __launch_bounds__(512) team_solve_kernel(const float* __restrict
     const int KK = K * K, ctr = KK - 1;
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
     const int b = blockIdx.x;
-    const bool ident = b >= C;                // CTAs C, C+1, ...: 32-column chunks of the identity (tap 0)
-    const int c0 = ident ? (b - C) * 32 : 0;  // first identity column of this CTA
+    // CTAs C .. CP_-1 (operand form only): channels that pad the operand, zeros; CTAs CP_, CP_+1, ...: 32-column chunks of the
+    // identity (tap 0)
+    const bool ident = b >= CP_;
+    const int c0 = ident ? (b - CP_) * 32 : 0;  // first identity column of this CTA
     const int NC = ident ? min(32, C - c0) : KK;   // right-hand-side columns
     const int NCB = KK > 32 ? KK : 32, YS = NCB | 1;
     float* Tt = sm;                           // [C][CP]   Tt[pa*CP + pi] = T[row at position pi][row at position pa], pi > pa
     float* invd = Tt + C * CP;                // [C]       1 / T[p][p], by position
     float* RHS = invd + ((C + 3) & ~3);       // [C][NC]   by row index
     float* Y = RHS + C * NCB;                 // [C][YS]   solved rows, by row index
+    if (!ident && b >= C) {
+        const int chunk = b >> 3, j = b & 7, rk = chunk / NCH, cl = chunk - rk * NCH, KCP = K * CP_;
+        for (int e = tid; e < K * KCP; e += NT) {
+            const int dh = e / KCP, row = e - dh * KCP;
+            pack_operand(wop + (size_t)rk * wbytes + (size_t)((dh * NCH + cl) * 4) * KCP * 16, KCP, row, j, 0.f, three != 0);
+        }
+        return;
+    }
     auto idx = [&](int pos) { return BWD ? C - 1 - pos : pos; };              // position in solve order -> row index
 
     // every global load of the CTA is issued before the first shared-memory store that waits for one
@@ -177,30 +207,25 @@ __global__ void __launch_bounds__(512) team_solve_kernel(const float* __restrict
     // Tensor-core operand form instead (see tensor_kernels.cuh): per CTA rank r = chunk / NCH one block
     //   [dh][chunk % NCH][plane 0,1: tf32 hi | plane 2: bf16 remainder | plane 3: bf16 value][row = dw*C + a][16 bytes],
     // chunk = input channel / 8; the sign is flipped for every tap but tap 0.
-    const int KC = K * C;
+    const int KC = K * CP_;
     for (int col = warp; col < NC; col += nwarps) {
         if (!ident && col == ctr) continue;
         const int tap = ident ? 0 : KK - 1 - col, ci = ident ? c0 + col : b;
         const int chunk = ci >> 3, j = ci & 7, rk = chunk / NCH, cl = chunk - rk * NCH;
         const int dh = tap / K, dw = tap - dh * K;
         unsigned char* blk = wop + (size_t)rk * wbytes + (size_t)((dh * NCH + cl) * 4) * KC * 16;
-        for (int a = lane; a < C; a += 32) {
-            const float y = Y[a * YS + col];
-            const float v = ident ? y : -y;
-            const float hi = tf32_hi(v);
-            const int row = dw * C + a;
-            *reinterpret_cast<float*>(blk + ((size_t)(j >> 2) * KC + row) * 16 + (j & 3) * 4) = hi;
-            *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)2 * KC + row) * 16 + j * 2) = __float2bfloat16_rn(v - hi);
-            *reinterpret_cast<__nv_bfloat16*>(blk + ((size_t)3 * KC + row) * 16 + j * 2) = __float2bfloat16_rn(v);
+        for (int a = lane; a < CP_; a += 32) {
+            const float y = a < C ? Y[a * YS + col] : 0.f;
+            pack_operand(blk, KC, dw * CP_ + a, j, ident ? y : -y, three != 0);
         }
     }
 }
 
 // Launch on `st` (grid: one CTA per input channel plus the identity chunks); cudaSuccess or the launch's error.
 inline cudaError_t team_solve_launch(bool bwd, const float* w, float* A, int C, int K, unsigned char* wop, int NCH,
-                                     unsigned wbytes, float* logdet_out, int HW, cudaStream_t st)
+                                     unsigned wbytes, int padded, bool three, float* logdet_out, int HW, cudaStream_t st)
 {
-    using Kern = void (*)(const float*, float*, int, int, unsigned char*, int, unsigned, float*, int);
+    using Kern = void (*)(const float*, float*, int, int, unsigned char*, int, unsigned, int, int, float*, int);
     Kern kern = nullptr;
     switch (team_solve_ns(C) * 2 + (bwd ? 1 : 0)) {
     case 2: kern = team_solve_kernel<false, 1>; break;
@@ -218,7 +243,7 @@ inline cudaError_t team_solve_launch(bool bwd, const float* w, float* A, int C, 
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
     }
-    kern<<<C + (C + 31) / 32, 512, sm, st>>>(w, A, C, K, wop, NCH, wbytes, logdet_out, HW);
+    kern<<<padded + (C + 31) / 32, 512, sm, st>>>(w, A, C, K, wop, NCH, wbytes, padded, three ? 1 : 0, logdet_out, HW);
     return cudaGetLastError();
 }
 

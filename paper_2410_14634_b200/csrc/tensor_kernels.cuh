@@ -44,8 +44,9 @@ struct TensorParams {
     const float* rhs;            // y (forward) or grad_x (backward), [B][C][H][W]
     float* out;                  // x or grad_y
     const unsigned char* wop;    // packed kernel: [R][wbytes]
-    int B, C, H, W, K;
-    int R, I, HP, S, ngroups, ncl, rot;
+    int B, C, H, W, K;           // C: channels in memory (the kernel's own count is this rounded up to eight)
+    int bulk;                    // slices of the images start on 16-byte boundaries: staged by bulk copies
+    int R, I, S, ngroups, ncl, rot;
     unsigned tmem_cols, wbytes, off_stage, off_x, off_y, off_recv, off_bar, stage_img;
 };
 
@@ -103,19 +104,93 @@ __device__ __forceinline__ void store_operand_row(unsigned char* chunk_base, int
     *reinterpret_cast<uint4*>(chunk_base + ((size_t)3 * rows + row) * 16) = lo;     // pairs with bf(w)
 }
 
+// The same with three bf16 terms per value (together 24 bits) in planes x0, x1, x2, x0 -- see mma_tap.
+__device__ __forceinline__ void split3(float v, float& a, float& b, float& c)
+{
+    a = __bfloat162float(__float2bfloat16_rn(v));
+    b = __bfloat162float(__float2bfloat16_rn(v - a));
+    c = v - a - b;
+}
+__device__ __forceinline__ void store_operand_row3(unsigned char* chunk_base, int rows, int row, const float (&v)[8])
+{
+    if (!INVCONV_CHECKED(row, rows, 101)) return;
+    float a[8], b[8], c[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) split3(v[j], a[j], b[j], c[j]);
+    const uint4 p0 = make_uint4(pack_bf16x2(a[0], a[1]), pack_bf16x2(a[2], a[3]), pack_bf16x2(a[4], a[5]), pack_bf16x2(a[6], a[7]));
+    *reinterpret_cast<uint4*>(chunk_base + ((size_t)0 * rows + row) * 16) = p0;
+    *reinterpret_cast<uint4*>(chunk_base + ((size_t)1 * rows + row) * 16) =
+        make_uint4(pack_bf16x2(b[0], b[1]), pack_bf16x2(b[2], b[3]), pack_bf16x2(b[4], b[5]), pack_bf16x2(b[6], b[7]));
+    *reinterpret_cast<uint4*>(chunk_base + ((size_t)2 * rows + row) * 16) =
+        make_uint4(pack_bf16x2(c[0], c[1]), pack_bf16x2(c[2], c[3]), pack_bf16x2(c[4], c[5]), pack_bf16x2(c[6], c[7]));
+    *reinterpret_cast<uint4*>(chunk_base + ((size_t)3 * rows + row) * 16) = p0;
+}
+
+// One contraction over the CTA's eight channels.  Descriptors: planes 0, 1 and planes 2, 3 of both operands; `plane` is the
+// weight operand's distance between planes in 16-byte units.
+//   two terms  : hi(w) hi(x) as a tf32 MMA, lo(w) bf(x) + bf(w) lo(x) as a bf16 MMA (19 bits)
+//   three terms: x0 w0 + x1 w1, x0 w1 + x1 w0, x2 w0 + x0 w2, three bf16 MMAs whose 16-deep contractions hold two products each;
+//                weight planes are w0, w1, w0, w2.  What is left out is below 2^-23 of a product: fp32 accuracy.
+template <bool T3>
+__device__ __forceinline__ void mma_tap(uint32_t d, uint64_t x01, uint64_t x23, uint64_t w01, uint64_t w23, uint32_t plane, uint32_t nbits, uint32_t acc)
+{
+    constexpr uint32_t tf = umma::make_idesc(umma::kFmtTF32, 0), bf = umma::make_idesc(umma::kFmtBF16, 0);
+    if constexpr (T3) {
+        umma::mma_bf16(d, x01, w01, bf | nbits, acc);
+        umma::mma_bf16(d, x01, w01 + plane, bf | nbits, 1u);
+        umma::mma_bf16(d, x23, w23, bf | nbits, 1u);
+    } else {
+        umma::mma_tf32(d, x01, w01, tf | nbits, acc);
+        umma::mma_bf16(d, x23, w23, bf | nbits, 1u);
+    }
+}
+// n slices of `slice` values, `sp` and `dp` apart, by 128 threads: one after the other where they are long; short ones as a single
+// run, so that the threads are kept busy and several loads are in flight.
+__device__ __forceinline__ void copy_slices(int n, int slice, int lt, const float* src, size_t sp, float* dst, size_t dp)
+{
+    if (slice >= 512) {
+        for (int ii = 0; ii < n; ++ii, src += sp, dst += dp)
+            for (int e = lt; e < slice; e += 8 * 128) {
+                float t[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (e + u * 128 < slice) t[u] = src[e + u * 128];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (e + u * 128 < slice) dst[e + u * 128] = t[u];
+            }
+        return;
+    }
+    int ii = slice > 0 ? lt / slice : n, r = lt - ii * slice;
+    while (ii < n) {
+        float t[4];
+        int at[4], im[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            im[u] = ii; at[u] = r;
+            if (ii < n) t[u] = src[ii * sp + r];
+            r += 128;
+            while (r >= slice) { r -= slice; ++ii; }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (im[u] < n) dst[im[u] * dp + at[u]] = t[u];
+    }
+}
+
 }  // namespace tensor_detail
 
-// CG = C / 16, K = kernel side.  NCH = 1 (eight contraction channels per CTA).
-template <int CG, int K>
+// R = CTAs of the cluster = channels / 8 (rounded up), K = kernel side, T3 = three-term products (see mma_tap).
+template <int R, int K, bool T3>
 __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(const TensorParams p)
 {
     using namespace tensor_detail;
-    constexpr int C = CG * 16;
     constexpr int CS = 8;
+    constexpr int C = R * CS;
     constexpr int S = 2 * (K - 1);
-    constexpr int R = C / CS;
+    constexpr int PG = (R + 1) / 2;             // peers per warpgroup of the exchange
     constexpr int KC = K * C;
-    constexpr int MAXSLOTS = 256 / C;
+    constexpr int MAXSLOTS = 256 / C > 0 ? 256 / C : 1;
     extern __shared__ __align__(128) unsigned char tsmem[];
     unsigned char* const smem = tsmem;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -174,46 +249,58 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
-    const size_t img_floats = (size_t)C * H * W;
-    const unsigned slice_bytes = (unsigned)(CS * H * W * sizeof(float));
+    const size_t img_floats = (size_t)p.C * H * W;
+    const int nch = min(CS, p.C - (int)rank * CS);                // channels of this CTA that exist in memory
+    const unsigned slice_bytes = (unsigned)(nch * H * W * sizeof(float));
 
     if (warp < 8) {
         // ------------------------------------------------ accumulators -> solved pixels
         // Two threads per accumulator lane: warpgroup wg = warp / 4 takes the partial sums of the peers
-        // wg*CG .. wg*CG+CG-1 (8 columns each) and finishes channels 4wg .. 4wg+3 of this CTA's own eight.
+        // wg*PG .. wg*PG+PG-1 (8 columns each) and finishes channels 4wg .. 4wg+3 of this CTA's own eight.
         const int wg = warp >> 2;
         const int m = tid & 127, h = m / I, i = m - h * I;
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         // where this lane's partial sums land in each peer, and the peer's arrival barrier (buffer 0)
-        uint32_t remote_row[CG], remote_bar[CG];
+        uint32_t remote_row[PG], remote_bar[PG];
 #pragma unroll
-        for (int q = 0; q < CG; ++q) {
-            const int pr = wg * CG + q;
+        for (int q = 0; q < PG; ++q) {
+            const int pr = wg * PG + q < R ? wg * PG + q : R - 1;
             const int slot = (int)rank < pr ? (int)rank : (int)rank - 1;
             remote_row[q] = cluster_map_u32(smem_u32(s_recv + (size_t)slot * 128 * CS + (size_t)m * 4), (uint32_t)pr);
             remote_bar[q] = cluster_map_u32(smem_u32(rbar), (uint32_t)pr);
         }
         const uint32_t own_col = rank * CS + wg * 4;
         unsigned nd = 0;            // diagonals processed so far (all groups): buffer = nd & 1, phase = (nd >> 1) & 1
+        unsigned nx = 0;            // the same for the operand buffers, which with three terms take a diagonal of zeros ahead of each group
         unsigned ng = 0;            // groups processed so far
         for (int g = cluster_id; g < p.ngroups; g += p.ncl, ++ng) {
             const int img = g * I + i;
             const bool img_ok = img < p.B;
+            if constexpr (T3) {
+                unsigned char* xb = s_x + (nx & 1) * xbuf_bytes + (size_t)(HALO + m) * 16 + wg * 8;
+                if (ng) {
+#pragma unroll
+                    for (int pl = 0; pl < 4; ++pl) *reinterpret_cast<uint2*>(xb + (size_t)pl * ROWS * 16) = make_uint2(0u, 0u);
+                    fence_proxy_async();
+                }
+                mbar_arrive(xfull + (nx & 1));
+                ++nx;
+            }
             wait_bar(ybar, ng & 1, gave_up);
             int slot_d = 0;
-            for (int d = 0; d < D; ++d, ++nd) {
+            for (int d = 0; d < D; ++d, ++nd, ++nx) {
                 const unsigned b = nd & 1, ph = (nd >> 1) & 1;
                 wait_bar(accbar, nd & 1, gave_up);
                 umma::fence_after_sync();
-                uint32_t acc[CG][8], own[4];
+                uint32_t acc[PG][8], own[4];
                 const uint32_t col = (uint32_t)(slot_d * C);
                 (void)INVCONV_CHECKED(col + C - 1, p.tmem_cols, 105);
                 slot_d = slot_d + 1 == S ? 0 : slot_d + 1;
 #pragma unroll
-                for (int q = 0; q < CG; ++q) umma::tmem_ld8(lane_addr + col + (wg * CG + q) * 8, acc[q]);
+                for (int q = 0; q < PG; ++q) umma::tmem_ld8(lane_addr + col + (wg * PG + q < R ? wg * PG + q : R - 1) * 8, acc[q]);
                 umma::tmem_ld4(lane_addr + col + own_col, own);
 #pragma unroll
-                for (int q = 0; q < CG; ++q) umma::tmem_ld_fence(acc[q]);
+                for (int q = 0; q < PG; ++q) umma::tmem_ld_fence(acc[q]);
                 umma::tmem_ld_fence(own);
                 umma::fence_before_sync();
                 // partial sums of the other CTAs' output channels go to their owners
@@ -221,8 +308,8 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                 const int w = d - h;
                 const bool on_diag = h < H && w >= 0 && w < W;
 #pragma unroll
-                for (int q = 0; q < CG; ++q) {
-                    if (wg * CG + q != (int)rank && on_diag) {
+                for (int q = 0; q < PG; ++q) {
+                    if (wg * PG + q < R && wg * PG + q != (int)rank && on_diag) {
                         st_async_f32x4(remote_row[q] + boff, make_float4(__uint_as_float(acc[q][0]), __uint_as_float(acc[q][1]),
                                                                        __uint_as_float(acc[q][2]), __uint_as_float(acc[q][3])), remote_bar[q] + bbar);
                         st_async_f32x4(remote_row[q] + boff + 128 * 16, make_float4(__uint_as_float(acc[q][4]), __uint_as_float(acc[q][5]),
@@ -233,7 +320,7 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                 if (tid == 0) mbar_expect_tx(rbar + b, recv_bytes((d + 2) % D));   // arm the phase two diagonals ahead
                 // own channels 4wg .. 4wg+3: sum over the CTAs in rank order
                 const float* recv_b = s_recv + b * recv_buf_floats + wg * 128 * 4 + m * 4;
-                float4 pa[R - 1];
+                float4 pa[R > 1 ? R - 1 : 1];
 #pragma unroll
                 for (int sl = 0; sl < R - 1; ++sl)
                     pa[sl] = (on_diag && INVCONV_CHECKED((recv_b - s_recv) + (size_t)sl * 128 * CS + 3, 2 * recv_buf_floats, 102))
@@ -257,9 +344,19 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                     for (int j = 0; j < 4; ++j) v[j] = 0.f;
                 }
                 {   // this warpgroup's half of the operand row: tf32 plane wg, 8 bytes of each bf16 plane
-                    unsigned char* xb = s_x + b * xbuf_bytes;
+                    unsigned char* xb = s_x + (nx & 1) * xbuf_bytes;
                     const int row = HALO + m;
                     (void)INVCONV_CHECKED(row, ROWS, 101);
+                    if constexpr (T3) {
+                        float a0[4], a1[4], a2[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) split3(v[j], a0[j], a1[j], a2[j]);
+                        const uint2 p0 = make_uint2(pack_bf16x2(a0[0], a0[1]), pack_bf16x2(a0[2], a0[3]));
+                        *reinterpret_cast<uint2*>(xb + ((size_t)0 * ROWS + row) * 16 + wg * 8) = p0;
+                        *reinterpret_cast<uint2*>(xb + ((size_t)1 * ROWS + row) * 16 + wg * 8) = make_uint2(pack_bf16x2(a1[0], a1[1]), pack_bf16x2(a1[2], a1[3]));
+                        *reinterpret_cast<uint2*>(xb + ((size_t)2 * ROWS + row) * 16 + wg * 8) = make_uint2(pack_bf16x2(a2[0], a2[1]), pack_bf16x2(a2[2], a2[3]));
+                        *reinterpret_cast<uint2*>(xb + ((size_t)3 * ROWS + row) * 16 + wg * 8) = p0;
+                    } else {
                     float hi[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) hi[j] = tf32_hi(v[j]);
@@ -268,9 +365,10 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                         make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]));
                     *reinterpret_cast<uint2*>(xb + ((size_t)3 * ROWS + row) * 16 + wg * 8) =
                         make_uint2(pack_bf16x2(v[0] - hi[0], v[1] - hi[1]), pack_bf16x2(v[2] - hi[2], v[3] - hi[3]));
+                    }
                 }
                 fence_proxy_async();
-                mbar_arrive(xfull + b);
+                mbar_arrive(xfull + (nx & 1));
                 if (valid) {
                     const int hh = p.rot ? H - 1 - h : h, ww = p.rot ? W - 1 - w : w;
                     float* dst = s_stage + (size_t)i * p.stage_img + (size_t)(wg * 4) * H * W + (size_t)hh * W + ww;
@@ -297,11 +395,12 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
             const uint64_t wd_tf = umma::make_desc(smem_u32(s_w), wplane);
             const uint64_t wd_bf = umma::make_desc(smem_u32(s_w) + 2 * wplane, wplane);
             const uint32_t xbuf16 = xbuf_bytes >> 4, ybuf16 = ybuf_bytes >> 4;
-            constexpr uint32_t idesc_tf = umma::make_idesc(umma::kFmtTF32, 0), idesc_bf = umma::make_idesc(umma::kFmtBF16, 0);
+            constexpr uint32_t wp16 = wplane >> 4, bfd = umma::make_idesc(umma::kFmtBF16, 0);
             constexpr uint32_t cbits = ((uint32_t)C >> 3) << 17;
             const uint64_t w01_tf = wd_tf + (uint64_t)C, w01_bf = wd_bf + (uint64_t)C;                         // dh = 0, dw = 1
             const uint64_t w10_tf = wd_tf + (uint64_t)(4 * (wplane >> 4)), w10_bf = wd_bf + (uint64_t)(4 * (wplane >> 4));   // dh = 1, dw = 0
-            unsigned nd = 0, ny = 0;
+            const uint64_t wll = (uint64_t)((K - 1) * 4 * (wplane >> 4) + (K - 1) * C), wll_tf = wd_tf + wll, wll_bf = wd_bf + wll;   // dh = dw = K - 1
+            unsigned nx = 0, ny = 0;
             // taps (dh, a .. a+n-1) of the solved diagonal d in buffer b -> the slots of diagonals d+dh+a ...;
             // slot_d = d mod S.  Split where the slot ring wraps and at 256 accumulator columns.
             auto window = [&](unsigned b, int d, int slot_d, int dh, int a, int n) {
@@ -320,47 +419,80 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                     const uint32_t nbits = ((uint32_t)(c * C) >> 3) << 17;
                     if (!INVCONV_CHECKED((s0 + c) * C - 1, p.tmem_cols, 106) || !INVCONV_CHECKED(HALO - dh * I, ROWS - 127, 107) ||
                         !INVCONV_CHECKED((a + c) * C - 1, KC, 108)) break;
-                    umma::mma_tf32(dcol, atf, wd_tf + wrow + (uint32_t)(a * C), idesc_tf | nbits, 1u);
-                    umma::mma_bf16(dcol, abf, wd_bf + wrow + (uint32_t)(a * C), idesc_bf | nbits, 1u);
+                    mma_tap<T3>(dcol, atf, abf, wd_tf + wrow + (uint32_t)(a * C), wd_bf + wrow + (uint32_t)(a * C), wp16, nbits, 1u);
                     a += c; n -= c; s0 += c;
                     if (s0 >= S) s0 -= S;
                 }
             };
-            // rhs of the next diagonal (operand buffer ny & 1) through A_0 = tap (0,0): opens slot `slot`
+            // The rhs of diagonal `ny` (operand buffer ny & 1) through A_0 = tap (0,0).
+            //   two terms  : opens the slot, S diagonals ahead of its use.
+            //   three terms: every MMA rounds its accumulator towards zero, so the largest term, hi(rhs) hi(A_0), comes last: when it
+            //                came first, each later MMA cut off up to one unit in the last place of the finished sum (residual 8e-7
+            //                instead of 1.1e-7 at C = 96, k = 3).  The slot is opened by the tap that reaches furthest, the small
+            //                products go in ahead of the wait for the previous diagonal.  Costs 2 us of 51 at 64x24x16x16, and
+            //                more where the tensor pipe is the bound: two-term products, whose 2^-19 is the larger error, keep theirs.
+            auto rhs_wait = [&]() {
+                wait_bar(yfull + (ny & 1), (ny >> 1) & 1, gave_up);
+                umma::fence_after_sync();
+            };
             auto rhs_tap = [&](int slot) {
                 const unsigned b = ny & 1;
-                wait_bar(yfull + b, (ny >> 1) & 1, gave_up);
-                umma::fence_after_sync();
+                rhs_wait();
+                mma_tap<T3>(tmem + (uint32_t)(slot * C), yd_tf + b * ybuf16, yd_bf + b * ybuf16, wd_tf, wd_bf, wp16, cbits, 0u);
+                umma::commit(yfree + b);
+                ++ny;
+            };
+            auto rhs_low = [&](int slot) {
+                const unsigned b = ny & 1;
+                rhs_wait();
                 const uint32_t dcol = tmem + (uint32_t)(slot * C);
-                constexpr uint32_t nbits = ((uint32_t)C >> 3) << 17;
-                umma::mma_tf32(dcol, yd_tf + b * ybuf16, wd_tf, idesc_tf | nbits, 0u);
-                umma::mma_bf16(dcol, yd_bf + b * ybuf16, wd_bf, idesc_bf | nbits, 1u);
+                umma::mma_bf16(dcol, yd_tf + b * ybuf16, wd_tf + wp16, bfd | cbits, 1u);
+                umma::mma_bf16(dcol, yd_bf + b * ybuf16, wd_bf, bfd | cbits, 1u);
+            };
+            auto rhs_high = [&](int slot) {
+                const unsigned b = ny & 1;
+                umma::mma_bf16(tmem + (uint32_t)(slot * C), yd_tf + b * ybuf16, wd_tf, bfd | cbits, 1u);
                 umma::commit(yfree + b);
                 ++ny;
             };
             for (int g = cluster_id; g < p.ngroups; g += p.ncl) {
-                for (int t = 0; t < S && t < D; ++t) rhs_tap(t);
+                if constexpr (T3) {
+                    // the first S slots are opened with the zeros that stand in for the diagonal before the first
+                    wait_bar(xfull + (nx & 1), (nx >> 1) & 1, gave_up);
+                    umma::fence_after_sync();
+                    for (int t = 0; t < S && t < D; ++t)
+                        umma::mma_bf16(tmem + (uint32_t)(t * C), xd_tf + ((nx & 1) ? (uint64_t)xbuf16 : 0ull), wd_tf, bfd | cbits, 0u);
+                    ++nx;
+                    rhs_low(0);
+                    rhs_high(0);
+                } else {
+                    for (int t = 0; t < S && t < D; ++t) rhs_tap(t);
+                }
                 umma::commit(accbar);
                 int slot_d = 0;
-                for (int d = 0; d < D; ++d, ++nd) {
-                    const unsigned b = nd & 1;
-                    wait_bar(xfull + b, (nd >> 1) & 1, gave_up);
+                for (int d = 0; d < D; ++d, ++nx) {
+                    const unsigned b = nx & 1;
+                    const int next = slot_d + 1 == S ? 0 : slot_d + 1;
+                    if (T3 && d + 1 < D) rhs_low(next);
+                    wait_bar(xfull + b, (nx >> 1) & 1, gave_up);
                     umma::fence_after_sync();
+                    const uint64_t xo = b ? (uint64_t)xbuf16 : 0ull;
                     if (d + 1 < D) {       // taps (0,1) and (1,0): the next diagonal waits for these only
-                        const uint32_t dcol = tmem + (uint32_t)((slot_d + 1 == S ? 0 : slot_d + 1) * C);
-                        const uint64_t xo = b ? (uint64_t)xbuf16 : 0ull;
-                        umma::mma_tf32(dcol, xd_tf + xo, w01_tf, idesc_tf | cbits, 1u);
-                        umma::mma_bf16(dcol, xd_bf + xo, w01_bf, idesc_bf | cbits, 1u);
-                        umma::mma_tf32(dcol, xd_tf + xo - (uint64_t)I, w10_tf, idesc_tf | cbits, 1u);
-                        umma::mma_bf16(dcol, xd_bf + xo - (uint64_t)I, w10_bf, idesc_bf | cbits, 1u);
+                        const uint32_t dcol = tmem + (uint32_t)(next * C);
+                        mma_tap<T3>(dcol, xd_tf + xo, xd_bf + xo, w01_tf, w01_bf, wp16, cbits, 1u);
+                        mma_tap<T3>(dcol, xd_tf + xo - (uint64_t)I, xd_bf + xo - (uint64_t)I, w10_tf, w10_bf, wp16, cbits, 1u);
+                        if (T3) rhs_high(next);
                         umma::commit(accbar);
                     }
-                    if (d + S < D) rhs_tap(slot_d);
+                    if (!T3 && d + S < D) rhs_tap(slot_d);
                     if (K > 2) window(b, d, slot_d, 0, 2, K - 2);
-                    window(b, d, slot_d, 1, 1, K - 1);
+                    if (K > 2 || !T3) window(b, d, slot_d, 1, 1, K - 1);
 #pragma unroll
-                    for (int dh = 2; dh < K; ++dh) window(b, d, slot_d, dh, 0, K);
-                    slot_d = slot_d + 1 == S ? 0 : slot_d + 1;
+                    for (int dh = 2; dh < K; ++dh) window(b, d, slot_d, dh, 0, T3 && dh == K - 1 ? K - 1 : K);
+                    if (T3 && d + S < D)   // the last tap reaches S diagonals ahead: it opens the slot just drained
+                        mma_tap<T3>(tmem + (uint32_t)(slot_d * C), xd_tf + xo - (uint64_t)((K - 1) * I), xd_bf + xo - (uint64_t)((K - 1) * I),
+                                    wll_tf, wll_bf, wp16, cbits, 0u);
+                    slot_d = next;
                 }
             }
         }
@@ -378,10 +510,15 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
         }
         for (int g = cluster_id; g < p.ngroups; g += p.ncl, ++ng) {
             const int nimg = min(I, p.B - g * I);
-            if (lt == 0) {
-                mbar_expect_tx(ybar, (unsigned)nimg * slice_bytes);
-                for (int ii = 0; ii < nimg; ++ii)
-                    if (INVCONV_CHECKED((size_t)(g * I + ii) * img_floats + (size_t)(rank + 1) * CS * H * W - 1, (size_t)p.B * img_floats, 109))
+            if (!p.bulk) {
+                // slices off a 16-byte boundary: copied by the four warps
+                copy_slices(nimg, nch * H * W, lt, p.rhs + (size_t)g * I * img_floats + (size_t)rank * CS * H * W, img_floats, s_stage, (size_t)p.stage_img);
+                asm volatile("bar.sync 2, 128;" ::: "memory");
+                if (lt == 0) mbar_arrive(ybar);
+            } else if (lt == 0) {
+                mbar_expect_tx(ybar, nch > 0 ? (unsigned)nimg * slice_bytes : 0u);
+                for (int ii = 0; ii < nimg && nch > 0; ++ii)
+                    if (INVCONV_CHECKED((size_t)(g * I + ii) * img_floats + (size_t)(rank * CS + nch) * H * W - 1, (size_t)p.B * img_floats, 109))
                         bulk_g2s(s_stage + (size_t)ii * p.stage_img,
                                  p.rhs + (size_t)(g * I + ii) * img_floats + (size_t)rank * CS * H * W, slice_bytes, ybar);
             }
@@ -397,19 +534,24 @@ __global__ void __launch_bounds__(kTensorThreads, 1) tensor_wavefront_kernel(con
                     const float* src = s_stage + (size_t)i * p.stage_img + (size_t)hh * W + ww;
                     const bool inb = INVCONV_CHECKED((src - s_stage) + (size_t)(CS - 1) * H * W, (size_t)I * p.stage_img, 104);
 #pragma unroll
-                    for (int j = 0; j < CS; ++j) v[j] = inb ? src[(size_t)j * H * W] : 0.f;
+                    for (int j = 0; j < CS; ++j) v[j] = inb && j < nch ? src[(size_t)j * H * W] : 0.f;
                 } else {
 #pragma unroll
                     for (int j = 0; j < CS; ++j) v[j] = 0.f;
                 }
-                store_operand_row(s_y + b * ybuf_bytes, 128, m, v);
+                if constexpr (T3) store_operand_row3(s_y + b * ybuf_bytes, 128, m, v);
+                else store_operand_row(s_y + b * ybuf_bytes, 128, m, v);
                 fence_proxy_async();
                 mbar_arrive(yfull + b);
             }
             // the solved slice leaves once every diagonal has been written to the staging buffer
-            if (lt == 0) {
+            if (!p.bulk) {
                 wait_bar(xdone, ng & 1, gave_up);
-                for (int ii = 0; ii < nimg; ++ii)
+                copy_slices(nimg, nch * H * W, lt, s_stage, (size_t)p.stage_img, p.out + (size_t)g * I * img_floats + (size_t)rank * CS * H * W, img_floats);
+                asm volatile("bar.sync 2, 128;" ::: "memory");
+            } else if (lt == 0) {
+                wait_bar(xdone, ng & 1, gave_up);
+                for (int ii = 0; ii < nimg && nch > 0; ++ii)
                     bulk_s2g(p.out + (size_t)(g * I + ii) * img_floats + (size_t)rank * CS * H * W,
                              s_stage + (size_t)ii * p.stage_img, slice_bytes);
                 bulk_commit();

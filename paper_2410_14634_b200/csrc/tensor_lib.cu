@@ -9,52 +9,20 @@
 #include "common.cuh"
 #include "lib_internal.h"
 #include "team_kernels.cuh"      // team_solve_kernel: the kernel transform L^-1 W_delta
-#include "tensor_kernels.cuh"
+#include "tensor_inst.cuh"
 #include "gradw_tensor.cuh"
 #include "conv_tensor.cuh"
 
 using namespace invconv;
-
-namespace {
-
-template <int CG, int K>
-int launch_tensor_inst(const TensorPlan& pl, const TensorParams& prm, cudaStream_t st)
-{
-    auto kern = tensor_wavefront_kernel<CG, K>;
-    const int rc = invconv_internal::set_smem_limit(kern, pl.smem);
-    if (rc) return rc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pl.ncl * pl.R);
-    cfg.blockDim = dim3(kTensorThreads);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = st;
-    // Programmatic dependent launch: the CTAs set themselves up (barriers, tensor memory, the right-hand side)
-    // while the kernel transform still runs; they wait for it (griddepcontrol.wait) before reading its output.
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = pl.R; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, prm);
-    if (e != cudaSuccess) {
-        std::fprintf(stderr, "invconv: tensor launch failed: %s\n", cudaGetErrorString(e));
-        cudaGetLastError();
-        return INVCONV_CUDA_ERROR;
-    }
-    return invconv_internal::check_launch();
-}
-
-}  // namespace
 
 namespace invconv_internal {
 
 int tensor_launch(const TensorPlan& pl, bool bwd, const float* rhs, const float* w, float* out, Geom g,
                   float* A, unsigned char* wop, cudaStream_t st, float* logdet_out)
 {
-    if (((reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out)) & 15) != 0) return INVCONV_UNSUPPORTED;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     {
-        if (team_solve_launch(bwd, w, A, g.C, g.k, wop, pl.NCH, pl.wbytes, logdet_out, g.H * g.W, st) != cudaSuccess) {
+        if (team_solve_launch(bwd, w, A, g.C, g.k, wop, pl.NCH, pl.wbytes, pl.C, pl.three, logdet_out, g.H * g.W, st) != cudaSuccess) {
             cudaGetLastError();
             return INVCONV_CUDA_ERROR;
         }
@@ -64,16 +32,17 @@ int tensor_launch(const TensorPlan& pl, bool bwd, const float* rhs, const float*
     TensorParams prm;
     prm.rhs = rhs; prm.out = out; prm.wop = wop;
     prm.B = g.B; prm.C = g.C; prm.H = g.H; prm.W = g.W; prm.K = g.k;
-    prm.R = pl.R; prm.I = pl.I; prm.HP = pl.HP; prm.S = pl.S; prm.ngroups = pl.ngroups; prm.ncl = pl.ncl;
+    prm.bulk = aligned && (g.C * g.H * g.W) % 4 == 0 && ((g.C % 8) * g.H * g.W) % 4 == 0 ? 1 : 0;
+    prm.R = pl.R; prm.I = pl.I; prm.S = pl.S; prm.ngroups = pl.ngroups; prm.ncl = pl.ncl;
     prm.rot = bwd ? 1 : 0;
     prm.tmem_cols = pl.tmem_cols; prm.wbytes = pl.wbytes;
     prm.off_stage = pl.off_stage; prm.off_x = pl.off_x; prm.off_y = pl.off_y; prm.off_recv = pl.off_recv;
     prm.off_bar = pl.off_bar; prm.stage_img = pl.stage_img;
-#define X(CG_, K_) if (g.C == 16 * CG_ && g.k == K_) return launch_tensor_inst<CG_, K_>(pl, prm, st);
-    X(1, 2) X(1, 3) X(1, 4) X(1, 5) X(2, 2) X(2, 3) X(2, 4) X(2, 5)
-    X(3, 2) X(3, 3) X(3, 4) X(3, 5) X(4, 2) X(4, 3) X(4, 4) X(4, 5)
+#define X(R_, K_) if (!pl.three && pl.R == R_ && g.k == K_) return launch_tensor_inst<R_, K_, false>(pl, prm, st);
+    X(2, 2) X(2, 3) X(2, 4) X(2, 5) X(4, 2) X(4, 3) X(4, 4) X(4, 5)
+    X(6, 2) X(6, 3) X(6, 4) X(6, 5) X(8, 2) X(8, 3) X(8, 4) X(8, 5)
 #undef X
-    return INVCONV_UNSUPPORTED;
+    return invconv_internal::tensor3_launch(pl, prm, g.k, st);
 }
 
 int gradw_tensor_launch(const GradWTensorPlan& pl, const float* gy, const float* x, float* partials, Geom g, cudaStream_t st)
@@ -167,18 +136,6 @@ int tensor_bounds_info(int* info)
     (void)info;
     return INVCONV_UNSUPPORTED;
 #endif
-}
-
-int tensor_read_clear_status(int* status_out)
-{
-    int v = 0;
-    if (cudaMemcpyFromSymbol(&v, g_device_status, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return INVCONV_CUDA_ERROR; }
-    if (v != 0) {
-        const int zero = 0;
-        cudaMemcpyToSymbol(g_device_status, &zero, sizeof(int));
-    }
-    *status_out = v;
-    return INVCONV_OK;
 }
 
 }  // namespace invconv_internal

@@ -9,8 +9,9 @@ struct TensorPlan {
     bool ok = false;
     int R = 0;          // CTAs per cluster = C / (8 * NCH)
     int NCH = 0;        // 8-channel chunks of the contraction per CTA
-    int I = 0;          // images per group (128 lanes / HP)
-    int HP = 0;         // image rows padded to 8 or 16
+    int I = 0;          // images per group (lane = row * I + image, at most 128 lanes)
+    int C = 0;          // channels, padded
+    bool three = false; // three-term products
     int S = 0;          // accumulator slots
     int ngroups = 0, ncl = 0;
     unsigned tmem_cols = 0;
@@ -23,22 +24,35 @@ struct TensorPlan {
 
 constexpr int kTensorThreads = 416;     // warps 0-7: accumulators -> solved pixels; warp 8: MMA issue; warps 9-12: right-hand side
 
-inline TensorPlan plan_tensor(int B, int C, int H, int W, int K, size_t max_smem, int sms)
+// `three`: three-term products, any channel count (padded to a multiple of 16, up to 16 CTAs) and image alignment.
+inline TensorPlan plan_tensor(int B, int C, int H, int W, int K, size_t max_smem, int sms, bool three = false)
 {
     TensorPlan pl;
-    if (K < 2 || K > 5 || H > 16 || C % 16 != 0 || C > 64 || (H * W) % 4 != 0 || B < 1) return pl;
+    if (K < 2 || K > 5 || B < 1) return pl;
+    if (!three && (H > 16 || C % 16 != 0 || C > 64 || (H * W) % 4 != 0)) return pl;
+    if (three && (H > 32 || K == 4)) return pl;
+    pl.three = three;
+    pl.C = (C + 15) / 16 * 16;
     pl.NCH = 1;
-    pl.R = C / 8;
-    if (pl.R < 2 || pl.R > 8) return pl;
-    pl.HP = H <= 8 ? 8 : 16;
-    pl.I = 128 / pl.HP;
+    pl.R = pl.C / 8;
+    if (pl.R < 2 || pl.R > (three ? 12 : 8)) return pl;
+    // images per group: lane = row * I + image, 128 lanes
+    pl.I = three ? 128 / H : 128 / (H <= 8 ? 8 : 16);
+    if (pl.I > B) pl.I = three ? B : pl.I;
     pl.S = 2 * (K - 1);
-    if (pl.S * C > 512) return pl;
+    if (pl.S * pl.C > 512) return pl;
     unsigned cols = 32;
-    while (cols < (unsigned)(pl.S * C)) cols *= 2;
+    while (cols < (unsigned)(pl.S * pl.C)) cols *= 2;
     pl.tmem_cols = cols;
-    const int CS = 8 * pl.NCH, KC = K * C, ROWS = (K - 1) * pl.I + 128;
+    const int CS = 8 * pl.NCH, KC = K * pl.C, ROWS = (K - 1) * pl.I + 128;
     auto up = [](size_t v) { return (v + 127) & ~(size_t)127; };
+    // a staged slice of many long rows: fewer images in a group, as many as the memory holds
+    if (three) {
+        const size_t fixed = (size_t)K * K * pl.C * 64 + 8 * (size_t)((K - 1) * pl.I + 128) * 16 + 8 * 128 * 16 + 2 * (size_t)(pl.R - 1) * 128 * 32 + 1024;
+        const size_t image = sizeof(float) * (size_t)(8 * H * W + 4);
+        if (fixed + image > max_smem) return pl;
+        if ((size_t)pl.I * image > max_smem - fixed) pl.I = (int)((max_smem - fixed) / image);
+    }
     pl.wbytes = (unsigned)(K * pl.NCH * KC * 64);
     pl.stage_img = (unsigned)(CS * H * W + 4);
     size_t off = up(pl.wbytes);

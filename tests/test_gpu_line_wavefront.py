@@ -10,7 +10,7 @@ from paper_2410_14634_b200 import workloads
 pytestmark = pytest.mark.gpu
 
 SHAPES = [
-    (3, 1, 5, 7, 2), (2, 2, 33, 40, 3), (300, 2, 9, 6, 3), (3, 3, 64, 64, 5), (2, 3, 70, 9, 5), (2, 4, 130, 60, 5), (9, 4, 70, 132, 5), (3, 3, 256, 64, 3), (2, 12, 52, 36, 2), (3, 4, 64, 60, 11), (1, 4, 1, 33, 3),
+    (3, 1, 5, 7, 2), (2, 2, 33, 40, 3), (300, 2, 9, 6, 3), (3, 3, 64, 64, 5), (2, 3, 70, 9, 5), (2, 4, 130, 60, 5), (9, 4, 70, 132, 5), (3, 3, 256, 64, 3), (2, 3, 210, 50, 3), (2, 12, 52, 36, 2), (3, 4, 64, 60, 11), (1, 4, 1, 33, 3),
     (2, 4, 40, 1, 5), (5, 5, 7, 9, 3), (3, 6, 45, 51, 3), (2, 8, 31, 17, 2), (160, 8, 16, 16, 3), (2, 9, 13, 12, 5), (301, 12, 4, 5, 3),
     (3, 12, 36, 36, 3), (2, 12, 32, 32, 5), (4, 13, 12, 10, 3), (3, 16, 32, 30, 3), (2, 16, 9, 8, 2), (2, 1, 40, 36, 7), (2, 2, 20, 18, 9),
     (3, 3, 64, 48, 7), (2, 4, 42, 40, 9), (2, 3, 32, 32, 11), (2, 4, 50, 13, 11), (1, 1, 12, 8, 11),
